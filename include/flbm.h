@@ -40,12 +40,12 @@ typedef struct flbm_batch flbm_batch;
  * which makes the viscosity of extensional flow differ from that of shear; with the
  * deviators at the shear rate (Lambda_5 = Lambda_6 = Lambda_7..9) the variant has one
  * viscosity, and Lambda_4 is the bulk rate. Statistics report k_4..k_6 in this basis.
- * Step variants 3, 4 and 6 run as 2, 2 and 5 for it. Not available in batches.
+ * Not available in batches.
  * FLBM_D3Q19 is the reduced lattice of Sec. II-C ("Lattice-agnostic construction and the
  * D3Q19 example"): rest, axis and face-diagonal velocities (weights 1/3, 1/18, 1/36) in the
  * order of the first 19 D3Q27 velocities, the printed 19-mode basis and norms, Lambda_7..9
- * the shear rates, and the equilibrium whose central moments are (rho, 0, ..., 0). Step
- * variants 3, 4 and 6 run as 2, 2 and 5 for it. Not available in batches. */
+ * the shear rates, and the equilibrium whose central moments are (rho, 0, ..., 0). Not
+ * available in batches. */
 enum flbm_lattice { FLBM_D2Q9 = 0, FLBM_D3Q27 = 1, FLBM_D3Q27_ISO = 2, FLBM_D3Q19 = 3 };
 
 /* Storage of the deviations d_i = f_i - w_i * rho0 in device memory. All moment
@@ -221,19 +221,15 @@ int flbm_stats_noalloc(int lattice, const int64_t dims[3], int storage, int pari
 
 /*
  * Step-kernel variant (launch configuration only; every variant computes the same
- * update): 0 = default (2 when nx is even, else 1), 1 = one site per thread, 2 = two
- * sites per thread, 3 = two sites per thread with the noise generated in a rolled loop
- * (smaller code), 4 = a persistent kernel that prefetches each row's populations into
- * shared memory with bulk asynchronous copies (needs nx even, nx <= 512 and a
- * population row a multiple of 16 bytes; else it falls back to 2), 5 and 6 = 2 and 3
- * compiled for more resident blocks per SM to hide latency: five for the 3-D lattices
- * (at most 102 registers), eight for D2Q9 (at most 64); 7 and 8 = 5 and 2 with blocks of
- * four rows of 32 site pairs instead of one row of 128 (for rows shorter than 256 sites,
- * which leave most of a one-row block idle). Variants 2-8 fall back to 1 when nx is odd.
+ * update): 0 = default (chosen by size, storage and noise), 1 = one site per thread, 2..8 =
+ * two sites per thread with the sites flattened over the rows, so that every row length
+ * fills the warps; 2, 3, 4 and 8 form 64-bit offsets, 5, 6 and 7 32-bit ones (a plane of
+ * 4 GB or more always takes 64). flbm_get_step_variant reports 0 as 2, every choice as 1
+ * when nx is odd (two sites per thread run all the same, unless 1 was chosen), and 4 as 2
+ * unless nx is even, at most 512 and a row of populations a multiple of 16 bytes.
  * The environment variable FLBM_STEP_VARIANT, read by flbm_create, sets the initial
  * choice.
- * flbm_autotune times every applicable variant (7 and 8 only for nx < 256) over
- * trial_steps steps on a copy of the current state (restored afterwards: populations
+ * flbm_autotune times variants 1, 2 and 5 over trial_steps steps on a copy of the current state (restored afterwards: populations
  * and step count are unchanged), keeps the fastest for this context and caches the
  * choice per (GPU model, lattice, storage, nx parity, size class, noise on/off, rate
  * structure, collision model, nx < 256) for the process; when the environment variable
@@ -254,8 +250,7 @@ int flbm_get_step_variant(const flbm_ctx *ctx);
  * every non-conserved rate equal to omega it is the fluctuating BGK step of Sec. II-A:
  * f* = f + omega (f^eq - f) + zeta with zeta_i = w_i sum_v b_v^-1 M_vi phi_v eta_v
  * (Eq. Xi_pop). Available for FLBM_D2Q9 and FLBM_D3Q27 (FLBM_EINVAL otherwise), not for the
- * lattices of a batch (FLBM_ESTATE); step variants 1 and 2 only (others run as 2, odd nx as
- * 1). Statistics still report the central moments of the orthogonal basis. The model is
+ * lattices of a batch (FLBM_ESTATE); flbm_get_step_variant reports every variant but 1 as 2. Statistics still report the central moments of the orthogonal basis. The model is
  * saved in checkpoints. Takes effect at the next flbm_step.
  */
 enum flbm_collision { FLBM_COLLISION_CM = 0, FLBM_COLLISION_RAW = 1 };
@@ -426,7 +421,7 @@ size_t flbm_slab_required_bytes(int lattice, const int64_t dims[3], int64_t z_co
  * exchanges the halo, see flbm_slab_halo, around every step taken from an odd step count);
  * flbm_stats covers the owned planes only (sites = nx ny z_count; add slabs' sums to
  * combine); flbm_get/set_populations, flbm_save/load cover the whole local array, ghost
- * planes included; flbm_autotune is refused (FLBM_ESTATE); step variant 4 runs as 2.
+ * planes included; flbm_autotune is refused (FLBM_ESTATE).
  * Errors: FLBM_EINVAL for D2Q9, a plane range outside [0, nz) or a local array of 2^32
  * sites or more.
  */

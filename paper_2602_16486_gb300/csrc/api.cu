@@ -51,7 +51,6 @@ struct flbm_ctx {
   int variant = 0;  // enum StepVariant; 0 = default choice
   bool shear = false;  // rates follow the paper's structure (collide.cuh, SHEAR)
   bool iso = false;    // the isotropic D3Q27 variant (lattice FLBM_D3Q27_ISO)
-  int *d_status = nullptr;  // device status word of the pipelined kernel
   StepArgs args{};
   flbm_batch *owner = nullptr;  // set for a lattice of a batch (borrowed handle)
   bool params_changed = false;  // a lattice of a batch reloaded its parameters
@@ -147,16 +146,30 @@ void fill_args(flbm_ctx *c) {
   StepArgs &a = c->args;
   a.f = c->f;
   a.plane = c->N;
+  for (int i = 0; i < 27; ++i)
+    a.pop[i] = static_cast<char *>(c->f) + size_t(i < c->Q ? i : 0) * size_t(c->N) * storage_bytes(c->storage);
   a.nx = int(c->dims[0]);
   a.ny = int(c->dims[1]);
   a.nz = int(c->dims[2]);
   a.rho0 = float(c->rho0);
-  a.status = c->d_status;
   a.z_lo = c->slab ? 1 : 0;
   a.nz_grid = c->slab ? int(c->z_count) : a.nz;
   // Global index of local site 0: nx ny (z_begin - 1), taken mod 2^32 (the ghost plane
   // below z_begin = 0 wraps; it is never updated).
   a.site_base = c->slab ? uint32_t(uint64_t(int64_t(c->dims[0] * c->dims[1]) * (c->z_begin - 1))) : 0u;
+  // The same range as flat sites and as pair slots (pair.cuh).
+  const uint64_t row = uint64_t(a.nx), rows = uint64_t(a.ny) * uint64_t(a.nz_grid);
+  a.first = uint32_t(row * uint64_t(a.ny) * uint64_t(a.z_lo));
+  a.count = uint32_t(row * rows);
+  a.slots[0] = uint32_t((row * rows + 1) / 2);
+  a.slots[1] = uint32_t((row + 1) / 2 * rows);
+  a.aligned[0] = c->N % 2 == 0 && a.first % 2 == 0 && a.count % 2 == 0;
+  a.aligned[1] = row % 2 == 0;
+  a.wide = uint64_t(c->N) * storage_bytes(c->storage) > 0xFFFFFFFFull;
+  batch_magic(uint32_t((a.nx + 1) / 2), &a.m_hp, &a.p_hp);
+  batch_magic(uint32_t(a.ny), &a.m_ny, &a.p_ny);
+  a.early = a.slots[0] > kEarlySlots;
+  a.sqrt_kbt = float(std::sqrt(c->kBT));
   a.key0 = uint32_t(c->seed);
   a.key1 = uint32_t(c->seed >> 32);
   for (int r = 0; r < 10; ++r) {  // Weyl key schedule of Philox4x32 (Salmon et al., SC'11)
@@ -168,11 +181,13 @@ void fill_args(flbm_ctx *c) {
     a.phc[v] = 0.0f;
     a.om_t[v] = 0.0f;
     a.phc_t[v] = 0.0f;
+    a.amp[v] = 0.0f;
   }
   for (int v = c->D + 1; v < c->Q; ++v) {
     const double L = c->lambda[v];
     a.om[v] = float(1.0 - L);
     a.phc[v] = float(std::sqrt(c->kBT * L * (2.0 - L) * mode_bnorm_lattice(c->lattice, v) * 3.0));
+    a.amp[v] = float(std::sqrt(L * (2.0 - L)));
     // Scales are powers of two: the products are exact.
     a.om_t[v] = a.om[v] * mode_tile_scale(c->lattice, v);
     a.phc_t[v] = a.phc[v] * mode_tile_scale(c->lattice, v);
@@ -196,7 +211,6 @@ void release(flbm_ctx *c) {
   if (c->d_ring) cudaFree(c->d_ring);
   if (c->d_stage) cudaFree(c->d_stage);
   if (c->d_sites) cudaFree(c->d_sites);
-  if (c->d_status) cudaFree(c->d_status);
   if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
   delete c;
 }
@@ -289,17 +303,23 @@ int enqueue_stats(flbm_ctx *c, double *acc_dev) {
   return FLBM_OK;
 }
 
-// Variant actually launched: the choice, or the default (two sites per thread where nx
-// is even, else one site per thread); the pipelined choice falls back where it does not
-// apply.
+// Whether variant 4 takes the box (even rows of at most 512 sites, of whole 16-byte words,
+// two stages of which fit in shared memory); otherwise the choice counts as 2.
+bool long_rows_fit(const flbm_ctx *c) {
+  const size_t row = size_t(c->dims[0]) * storage_bytes(c->storage);
+  return c->dims[0] % 2 == 0 && c->dims[0] <= 512 && row % 16 == 0 &&
+         2 * size_t(c->D == 3 ? 27 : 9) * row + 16 <= 232448;
+}
+
+// The variant as flbm_get_step_variant reports it: the choice, or the default (two sites per
+// thread where nx is even, else one).
 int resolve_variant(const flbm_ctx *c) {
   if (c->model == FLBM_COLLISION_RAW)  // raw-moment kernels: one site or two per thread
     return c->dims[0] % 2 != 0 || c->variant == kStepOneSite ? int(kStepOneSite) : int(kStepPair);
-  const bool pipe = pipe_applicable(c->D, c->storage, int(c->dims[0]));
   int v = c->variant;
   if (v == kStepAuto) v = kStepPair;
-  if (v == kStepPipelined && (!pipe || c->slab)) v = kStepPair;  // the pipelined kernel walks whole boxes
-  if (pair_variants_only(c->lattice)) {  // unrolled two-site kernels only
+  if (v == kStepPipelined && (!long_rows_fit(c) || c->slab)) v = kStepPair;
+  if (pair_variants_only(c->lattice)) {
     if (v == kStepPairRolled || v == kStepPipelined) v = kStepPair;
     if (v == kStepPairRolledOcc) v = kStepPairOcc;
   }
@@ -307,15 +327,14 @@ int resolve_variant(const flbm_ctx *c) {
   return v;
 }
 
-// Reads and clears the device status word (after a synchronisation).
-int check_status(flbm_ctx *c) {
-  int h = 0;
-  FLBM_CUDA(cudaMemcpy(&h, c->d_status, sizeof(int), cudaMemcpyDeviceToHost));
-  if (h != 0) {
-    FLBM_CUDA(cudaMemset(c->d_status, 0, sizeof(int)));
-    return fail(FLBM_ETIMEOUT, "a bounded wait in the pipelined step kernel gave up; the state is not valid");
-  }
-  return FLBM_OK;
+// The variant launched. One site per thread only where it was asked for (the pair kernels take
+// every row length). The default is the form with 32-bit offsets but for large noisy FP32
+// D3Q27 boxes, which are bound by DRAM and stream better with 64-bit ones (256^3: 0.549 against
+// 0.557 ms; below the size of `early` 64^3: 10.3 against 10.0 us, 16-bit 256^3: 0.534 against 0.522).
+int launch_variant(const flbm_ctx *c) {
+  if (c->variant != kStepAuto) return c->variant;
+  const bool dram = c->D == 3 && c->Q == 27 && c->storage == FLBM_FP32 && c->kBT > 0.0 && c->args.early;
+  return dram ? int(kStepPair) : int(kStepPairOcc);
 }
 
 struct CkptHeader {
@@ -401,8 +420,6 @@ int flbm_create_ex(flbm_ctx **out, int lattice, const int64_t dims[3], const dou
   const size_t acc_bytes = sizeof(double) * stats_record_len(c->Q);
   e = cudaMalloc(&c->d_acc, acc_bytes);
   if (e == cudaSuccess) e = cudaMallocHost(&c->h_acc, acc_bytes);
-  if (e == cudaSuccess) e = cudaMalloc(&c->d_status, sizeof(int));
-  if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, sizeof(int), c->stream);
   if (e != cudaSuccess) {
     cudaGetLastError();
     release(c);
@@ -463,9 +480,9 @@ int flbm_step(flbm_ctx *c, int64_t n) {
     c->args.step_lo = uint32_t(uint64_t(c->step));
     c->args.step_hi = uint32_t(uint64_t(c->step) >> 32);
     if (c->model == FLBM_COLLISION_RAW)
-      FLBM_CUDA(launch_step_raw(c->D, c->storage, resolve_variant(c), int(c->step & 1), noise, c->args, c->stream));
+      FLBM_CUDA(launch_step_raw(c->D, c->storage, launch_variant(c), int(c->step & 1), noise, c->args, c->stream));
     else
-      FLBM_CUDA(launch_step(c->lattice, c->storage, resolve_variant(c), int(c->step & 1), noise, c->shear,
+      FLBM_CUDA(launch_step(c->lattice, c->storage, launch_variant(c), int(c->step & 1), noise, c->shear,
                             c->args, c->stream));
     ++c->step;
   }
@@ -483,8 +500,6 @@ int flbm_stats(flbm_ctx *c, flbm_stats_t *out) {
   FLBM_CUDA(cudaMemcpyAsync(c->h_acc, c->d_acc, sizeof(double) * stats_record_len(c->Q),
                             cudaMemcpyDeviceToHost, c->stream));
   FLBM_CUDA(cudaStreamSynchronize(c->stream));
-  const int status = check_status(c);
-  if (status != FLBM_OK) return status;
   fill_stats(c, c->h_acc, c->step, out);
   return stats_result(out, (long long)c->step);
 }
@@ -778,16 +793,7 @@ int flbm_autotune(flbm_ctx *c, int trial_steps, int *chosen) {
       st = fail(FLBM_ECUDA, "autotune set-up: %s", cudaGetErrorString(cudaGetLastError()));
       break;
     }
-    const int candidates[8] = {kStepOneSite, kStepPair,    kStepPairRolled,  kStepPipelined,
-                               kStepPairOcc, kStepPairRolledOcc, kStepPairOccRows, kStepPairRows};
-    for (int v : candidates) {
-      if (pair_variants_only(c->lattice) &&
-          (v == kStepPairRolled || v == kStepPipelined || v == kStepPairRolledOcc))
-        continue;
-      // Blocks of four rows only where a row is shorter than a one-row block's 256 sites.
-      if ((v == kStepPairOccRows || v == kStepPairRows) && c->dims[0] >= 2 * kStepBlock) continue;
-      if (v != kStepOneSite && c->dims[0] % 2 != 0) continue;
-      if (v == kStepPipelined && !pipe_applicable(c->D, c->storage, int(c->dims[0]))) continue;
+    for (int v : {int(kStepOneSite), int(kStepPair), int(kStepPairOcc)}) {
       c->variant = v;
       if ((st = flbm_step(c, 2)) != FLBM_OK) break;  // warm-up (both parities)
       cudaEventRecord(e0, c->stream);
@@ -837,7 +843,7 @@ int flbm_sync(flbm_ctx *c) {
   if (!c) return fail(FLBM_EINVAL, "ctx is NULL");
   DeviceGuard g(c->device);
   FLBM_CUDA(cudaStreamSynchronize(c->stream));
-  return check_status(c);
+  return FLBM_OK;
 }
 
 const char *flbm_last_error(void) { return g_last_error.c_str(); }
@@ -934,7 +940,7 @@ int batch_params(flbm_batch *b) {
     const int ref = c->D == 3 ? 7 : 5;  // a shear mode with b = 1/9
     L.sqrt_kbt = float(std::sqrt(c->kBT));
     L.om_shear = a.om[ref];
-    L.phc_shear = a.phc[ref];
+    L.amp_shear = a.amp[ref];
     for (int v = 0; v < 27; ++v) {
       rates[size_t(i) * 54 + size_t(v)] = a.om_t[v];  // the collision's (tile-scaled) constants
       rates[size_t(i) * 54 + 27 + size_t(v)] = a.phc_t[v];
@@ -942,9 +948,9 @@ int batch_params(flbm_batch *b) {
     // The shear form needs the paper's structure and one rate shared by the shear modes.
     bool ok = c->shear;
     if (c->D == 3)
-      ok = ok && a.om[8] == a.om[7] && a.om[9] == a.om[7] && a.phc[8] == a.phc[7] && a.phc[9] == a.phc[7];
+      ok = ok && a.om[8] == a.om[7] && a.om[9] == a.om[7] && a.amp[8] == a.amp[7] && a.amp[9] == a.amp[7];
     else
-      ok = ok && a.om[4] == a.om[5] && a.phc[4] == 2.0f * a.phc[5];
+      ok = ok && a.om[4] == a.om[5] && a.amp[4] == a.amp[5];
     if (!ok) b->shear = false;
     c->params_changed = false;
   }

@@ -1,5 +1,4 @@
-// Bulk asynchronous copies (the TMA engine's cp.async.bulk, global -> shared) tracked
-// by shared-memory mbarriers, written as inline PTX (PTX ISA: mbarrier, cp.async.bulk).
+// Shared-memory mbarriers, written as inline PTX (PTX ISA: mbarrier).
 // Every wait is bounded: after kSpinLimit polls it reports failure instead of hanging.
 #pragma once
 
@@ -17,25 +16,9 @@ __device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");
 }
 
-// Makes initialised mbarriers visible to the async proxy (the bulk-copy engine).
+// Makes initialised mbarriers visible to the async proxy.
 __device__ __forceinline__ void fence_mbar_init() {
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-}
-
-// One arrival that also announces `bytes` of transactions the copies will complete.
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes)
-               : "memory");
-}
-
-// Contiguous copy of `bytes` (multiple of 16, both addresses 16-byte aligned) from global
-// to this CTA's shared memory; completion is counted on `bar`.
-__device__ __forceinline__ void bulk_copy_g2s(void *dst, const void *src, uint32_t bytes, uint64_t *bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-          smem_addr(dst)),
-      "l"(src), "r"(bytes), "r"(smem_addr(bar))
-      : "memory");
 }
 
 __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {

@@ -35,6 +35,7 @@
 
 #include "collide.cuh"
 #include "internal.h"
+#include "pair.cuh"
 
 namespace flbm {
 namespace {
@@ -47,12 +48,16 @@ template <int D, bool SHEAR, bool ROLLED>
 __device__ __forceinline__ void collide_lattice(float2 (&F)[3][3][3], const BatchLattice &L, const float *rates,
                                                 uint32_t s0, uint32_t dsite, uint32_t step_lo, uint32_t step_hi) {
   const KeyBase keys{L.key0, L.key1};
-  if (SHEAR)
-    collide_rates<D, true, float2, ROLLED, true>(F, L.rho0, ShearRates<D>{L.sqrt_kbt, L.om_shear, L.phc_shear},
-                                                 s0, step_lo, step_hi, keys, dsite);
-  else
-    collide_rates<D, true, float2, ROLLED, false>(F, L.rho0, ArrayRates{rates, rates + 27}, s0, step_lo, step_hi,
-                                                  keys, dsite);
+  float2 n[Noisy<D>::count];
+  if (SHEAR) {
+    const ShearRates<D> r{L.sqrt_kbt, L.om_shear, L.amp_shear};
+    noise_modes<D, true, false, 0, Noisy<D>::blocks>(n, r, s0, step_lo, step_hi, keys, dsite);
+    collide_rates<D, true, float2, true>(F, L.rho0, r, n);
+  } else {
+    const ArrayRates r{rates, rates + 27, nullptr, 0.0f};
+    noise_modes<D, false, false, 0, Noisy<D>::blocks>(n, r, s0, step_lo, step_hi, keys, dsite);
+    collide_rates<D, true, float2, false>(F, L.rho0, r, n);
+  }
 }
 
 // Pair slots of lattice L: row r = y + ny z holds ceil(nx / 2) slots, and slot j of it
@@ -61,10 +66,6 @@ __device__ __forceinline__ void collide_lattice(float2 (&F)[3][3][3], const Batc
 // accesses stay contiguous for every nx.
 __device__ __forceinline__ uint32_t pair_slots(const BatchLattice &L) {
   return (uint32_t)((L.nx + 1) >> 1) * (uint32_t)L.ny * (uint32_t)L.nz;
-}
-
-__device__ __forceinline__ uint32_t udiv_magic(uint32_t x, uint32_t m, int p) {
-  return (uint32_t)(((unsigned long long)x * m) >> p);
 }
 
 // Row coordinates of pair slot `slot` (32-bit arithmetic: every site index is < 2^32, so

@@ -181,37 +181,26 @@ __device__ __forceinline__ void d3q19_macros(const T (&F)[19], float rho0, T (&r
 
 // The collision of one site (float) or two (float2); on return F holds the post-collision
 // deviations. SHEAR: the paper's rates (1 except the shear modes 7-9), so only k_7..9 are
-// formed. om_v = 1 - Lambda_v, phc_v = sqrt(kBT Lambda_v (2 - Lambda_v) b_v / cs^2).
-template <bool NOISE, typename T, bool SHEAR, typename K>
-__device__ __forceinline__ void collide19(T (&F)[19], float rho0, const float *om, const float *phc, uint32_t site0,
-                                          uint32_t step_lo, uint32_t step_hi, const K &keys, uint32_t dsite = 1) {
+// formed. om_v = 1 - Lambda_v; n: the noise amplitudes of noise_modes (collide.cuh).
+template <bool NOISE, typename T, bool SHEAR>
+__device__ __forceinline__ void collide19(T (&F)[19], float rho0, const ArrayRates &rates,
+                                          const T (&n)[Noisy<19>::count]) {
   T r[19], rho, ux, uy, uz;
   d3q19_macros(F, rho0, r, rho, ux, uy, uz);
   const T jx = r[1], jy = r[2], jz = r[3], drho = r[0];
+  const T srho = NOISE ? noise_scale<SHEAR>(rho, rates) : rho;
   if (SHEAR) {
-    T k7, k8, k9;
-    d3q19_shear_central(r, rho, ux, uy, uz, k7, k8, k9);
+    T k[3];
+    d3q19_shear_central(r, rho, ux, uy, uz, k[0], k[1], k[2]);
 #pragma unroll
-    for (int v = 4; v < 19; ++v) r[v] = splat<T>(0.0f);
-    r[7] = vmul(splat<T>(om[7]), k7);
-    r[8] = vmul(splat<T>(om[8]), k8);
-    r[9] = vmul(splat<T>(om[9]), k9);
+    for (int v = 4; v < 19; ++v) r[v] = NOISE ? vmul(srho, n[v - 4]) : splat<T>(0.0f);
+#pragma unroll
+    for (int v = 7; v < 10; ++v)
+      r[v] = relaxed<NOISE>(NOISE ? vmul(splat<T>(rates.amp(v)), srho) : srho, n[v - 4], rates.om(v), k[v - 7]);
   } else {
     d3q19_central_lr(r, rho, ux, uy, uz);
 #pragma unroll
-    for (int v = 4; v < 19; ++v) r[v] = vmul(splat<T>(om[v]), r[v]);
-  }
-  if (NOISE) {
-  #pragma unroll
-    for (int blk = 0; blk < 4; ++blk) {
-      T z[4];
-      normals4_scaled<T>(site0, step_lo, step_hi, (uint32_t)blk, keys, rho, z, dsite);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int v = 4 + 4 * blk + j;
-        if (v < 19) r[v] = vfma(splat<T>(phc[v]), z[j], r[v]);
-      }
-    }
+    for (int v = 4; v < 19; ++v) r[v] = relaxed<NOISE>(srho, n[v - 4], rates.om(v), r[v]);
   }
   // The general rates keep more values live; they use the register-lean inverse.
   if (SHEAR)

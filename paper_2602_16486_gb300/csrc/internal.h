@@ -10,12 +10,17 @@
 
 namespace flbm {
 
-constexpr int kStepBlock = 128;   // threads per block of the step kernels (x direction)
+constexpr int kStepBlock = 128;   // threads per block of the step kernels
+// Pair slots from which a step launch is longer than two rounds of the GPU (152 SMs, five blocks
+// each): its blocks then read before they form any noise, and the launch before it has long
+// drained. Shorter launches overlap noise with that drain instead.
+constexpr uint32_t kEarlySlots = 2u * 152u * 5u * 128u;
 constexpr int kStatsBlock = 128;  // threads (= sites per tile) of the statistics kernel
 
 // Arguments of one fused step launch (passed by value, lives in the constant bank).
 struct StepArgs {
   void *f;            // populations (deviations), Q planes of `plane` elements
+  char *pop[27];      // the planes
   long long plane;    // nx * ny * nz
   int nx, ny, nz;
   float rho0;
@@ -27,11 +32,22 @@ struct StepArgs {
   // local site 0 (0 for a whole box), added to the local site index that keys the noise.
   int z_lo, nz_grid;
   uint32_t site_base;
-  int *status;        // device word: nonzero after a bounded wait gave up (pipelined kernel)
+  // The pair kernels' view of the same range (pair.cuh), by the parity of the step taken: its
+  // flat sites [first, first + count), pair slots, whether pairs move as one word, and the
+  // divisions by ceil(nx / 2) and ny (batch_magic).
+  uint32_t first, count;
+  uint32_t slots[2];
+  bool aligned[2];
+  bool wide;  // a plane of 4 GB or more: 64-bit offsets
+  uint32_t m_hp, m_ny;
+  int p_hp, p_ny;
   float om[27];       // 1 - Lambda_v (conserved modes: unused)
   float phc[27];      // sqrt(kBT Lambda_v (2 - Lambda_v) b_v / cs^2); phi_v = sqrt(rho) phc_v
   float om_t[27];     // om and phc times the mode's tile scale (lattice.cuh, tile_scale): the
   float phc_t[27];    // constants the D2Q9 / D3Q27 collision takes (isotropic modes 4-6: 1)
+  float amp[27];      // sqrt(Lambda_v (2 - Lambda_v))
+  float sqrt_kbt;
+  bool early;         // more blocks than two rounds of the GPU: read before forming any noise
 };
 
 // ---- batched ensembles (batch.cu) ----------------------------------------------------
@@ -47,7 +63,7 @@ struct BatchLattice {  // one lattice of a batch (FP32 storage); lives in the ke
   uint32_t dpp;    // D | p_hp << 8 | p_ny << 16 (lattice dimension and the shifts below)
   float rho0;
   uint32_t key0, key1;                  // noise key (seed)
-  float sqrt_kbt, om_shear, phc_shear;  // rates in the paper's structure (ShearRates)
+  float sqrt_kbt, om_shear, amp_shear;  // rates in the paper's structure (ShearRates)
   int tile0;                            // index of the lattice's first tile
   // Division by the row's pair-slot count and by ny as a multiply-high and a shift:
   // q = (x * m) >> p with p = 31 + ceil(log2 d), m = ceil(2^p / d), exact for x < 2^31.
@@ -103,25 +119,20 @@ cudaError_t launch_batch_steps(int form3, int threads3, int form2, int threads2,
 int stats_nacc(int Q);
 inline int stats_record_len(int Q) { return stats_nacc(Q) + 1; }  // + non-finite count
 
-// Step-kernel variants (the autotuner's search space; all compute the same update):
-// one site per thread; two sites per thread (nx even) with the noise loop unrolled or
-// rolled; or the bulk-copy pipelined persistent kernel (step_pipe.cu; needs
-// pipe_applicable). `shear` selects the specialisation for the paper's rate structure
-// (rate 1 for every non-conserved mode but the shear ones).
+// Step-kernel variants (include/flbm.h): one site per thread, or two with 64-bit offsets
+// (2, 3, 4, 8) or 32-bit ones (5, 6, 7).
 enum StepVariant {
   kStepAuto = 0,
   kStepOneSite = 1,
   kStepPair = 2,
   kStepPairRolled = 3,
   kStepPipelined = 4,
-  kStepPairOcc = 5,        // as 2, register cap for five blocks per SM (D3Q27)
-  kStepPairRolledOcc = 6,  // as 3, register cap for five blocks per SM (D3Q27)
-  kStepPairOccRows = 7,    // as 5, blocks of kRowBlockRows rows x 32 pair slots (short rows)
-  kStepPairRows = 8,       // as 2, blocks of kRowBlockRows rows x 32 pair slots (short rows)
+  kStepPairOcc = 5,
+  kStepPairRolledOcc = 6,
+  kStepPairOccRows = 7,
+  kStepPairRows = 8,
   kStepVariantMax = 8
 };
-constexpr int kRowBlockRows = 4;  // rows per block of variants 7 and 8 (one row per warp)
-bool pipe_applicable(int D, int storage, int nx);
 // lattice: the public lattice id (0 D2Q9, 1 D3Q27, 2 D3Q27 isotropic, 3 D3Q19).
 cudaError_t launch_step(int lattice, int storage, int variant, int parity, bool noise, bool shear,
                         const StepArgs &a, cudaStream_t s);
@@ -132,9 +143,7 @@ cudaError_t launch_step_iso(int storage, int variant, int parity, bool noise, bo
                             cudaStream_t s);
 cudaError_t launch_step_d3q19(int storage, int variant, int parity, bool noise, bool shear, const StepArgs &a,
                               cudaStream_t s);
-cudaError_t launch_step_pipelined(int D, int storage, int parity, bool noise, bool shear,
-                                  const StepArgs &a, cudaStream_t s);
-// The raw-moment collision (step_raw.cu): D 2 or 3, variants 1 (one site) and 2 (pairs).
+// The raw-moment collision (step_raw.cu): D 2 or 3.
 cudaError_t launch_step_raw(int D, int storage, int variant, int parity, bool noise, const StepArgs &a,
                             cudaStream_t s);
 // Statistics of the sites [site0, site0 + nsites) of the array (the whole box: 0, plane).

@@ -69,10 +69,10 @@ __device__ __forceinline__ uint4 philox4x32_10_ks(uint4 ctr, const K &keys) {
 // in (-pi, pi]. cos / sin come from the hardware approximations (__sincosf; absolute error
 // about 4e-7 on [-pi, pi]), which cost two instructions instead of a polynomial.
 //
-// The radius: u_a = (2 m_a + 1) 2^-24 with y = 2 m_a + 1 an odd integer below 2^24, so
-// -2 ln u_a = -2 (ln y - 24 ln 2). y converts to FP32 exactly; the argument reduction
-// of Cody & Waite (Software Manual for the Elementary Functions, 1980) writes y = 2^k x
-// with x in [sqrt(1/2), sqrt(2)), and ln x = 2 atanh(s) = 2 (s + s^3/3 + ... + s^9/9),
+// The radius: u_a = (2 m_a + 1) 2^-24 is formed exactly from the word's top 23 bits (1 + m 2^-23
+// assembled by one funnel shift, minus 1 - 2^-24). The argument reduction of Cody & Waite
+// (Software Manual for the Elementary Functions, 1980) writes u_a = 2^k x with x in
+// [sqrt(1/2), sqrt(2)), and ln x = 2 atanh(s) = 2 (s + s^3/3 + ... + s^9/9),
 // s = (x - 1)/(x + 1), |s| < 0.172 (truncation below 1e-9 relative). x - 1 is exact,
 // so the result keeps its relative accuracy as u_a -> 1, where r -> 0 (a hardware
 // logarithm has an absolute error there that exceeds the value). Checked against the FP64
@@ -80,64 +80,60 @@ __device__ __forceinline__ uint4 philox4x32_10_ks(uint4 ctr, const K &keys) {
 constexpr float kAngleScale = 0x1p-32f * 6.28318530717958647692f;  // 2 pi 2^-32
 constexpr float kAngleOffset = 0x1p-23f * 3.14159265358979323846f;  // pi 2^-23 = 2 pi 2^-24
 
-// Four normals of Philox block `blk` for each lane's site (lane l: site0 + l * dsite),
-// each multiplied by sqrt(rho) of its lane: the radius is taken as sqrt(-2 rho ln u_a)
-// (hardware square root, PTX sqrt.approx.ftz) in one product and one root per lane.
-template <typename T, typename K>
-__device__ __forceinline__ void normals4_scaled(uint32_t site0, uint32_t step_lo, uint32_t step_hi,
-                                                uint32_t blk, const K &keys, T rho, T (&z)[4],
-                                                uint32_t dsite = 1) {
+// Words of Philox block `blk` for each lane's site (lane l: site0 + l * dsite).
+template <int L, typename K>
+__device__ __forceinline__ void philox_lanes(uint32_t site0, uint32_t step_lo, uint32_t step_hi, uint32_t blk,
+                                             const K &keys, uint32_t dsite, uint4 (&w)[L]) {
+#pragma unroll
+  for (int l = 0; l < L; ++l)
+    w[l] = philox4x32_10_ks(make_uint4(site0 + uint32_t(l) * dsite, step_lo, step_hi, blk), keys);
+}
+
+// The Box-Muller pair of words (wa, wb): radius r = sqrt(V (-2 ln u_a)) and the cosine and
+// sine of the angle. V (a variance, compile-time when it is a literal) costs nothing: it
+// scales the constants of the logarithm. The series of -2 ln x / s = -4 atanh(s) / s in s^2 is
+// the minimax cubic on [0, 0.02944] (Remez exchange; relative error 7e-10, against the Taylor
+// quartic's 8e-8 s-dependent tail at one more multiply-add: the FP32 result is the same to its
+// rounding, 2.5e-7 over all 2^23 codes for both).
+template <typename T>
+__device__ __forceinline__ void box_muller(const uint32_t (&wa)[Lanes<T>::n], const uint32_t (&wb)[Lanes<T>::n],
+                                           double V, T &rad, T &c, T &sn) {
   constexpr int L = Lanes<T>::n;
-  float ang[L][2];
-  uint32_t wav[L][2];
+  T f, x, kf, ang;
 #pragma unroll
   for (int l = 0; l < L; ++l) {
-    const uint4 w = philox4x32_10_ks(make_uint4(site0 + uint32_t(l) * dsite, step_lo, step_hi, blk), keys);
-    wav[l][0] = w.x;
-    wav[l][1] = w.z;
-    ang[l][0] = fmaf((float)(int)w.y, kAngleScale, kAngleOffset);
-    ang[l][1] = fmaf((float)(int)w.w, kAngleScale, kAngleOffset);
+    set_lane(f, l, __uint_as_float(__funnelshift_r(wa[l], 0x7Fu, 9)));  // 1 + m 2^-23
+    set_lane(ang, l, (float)(int)wb[l]);
   }
+  const T u = vadd(f, splat<T>(-0x1.fffffep-1f));  // (m + 1/2) 2^-23, exact
 #pragma unroll
-  for (int p = 0; p < 2; ++p) {
-    T x, kf;
+  for (int l = 0; l < L; ++l) {
+    // bits(u) - bits(sqrt(1/2)): the sign and exponent field is k 2^23 (an arithmetic mask; no
+    // overflow for u in (0, 1)), and subtracting it from u's exponent gives x.
+    const uint32_t b = __float_as_uint(lane(u, l));
+    const uint32_t e = (b - 0x3F3504F3u) & 0xFF800000u;
+    set_lane(x, l, __uint_as_float(b - e));
+    set_lane(kf, l, (float)(int)e);  // k 2^23, exact
+  }
+  const T t = vadd(x, splat<T>(-1.0f));
+  const T d = vadd(x, splat<T>(1.0f));
+  T rd;
 #pragma unroll
-    for (int l = 0; l < L; ++l) {
-      // ix = bits(y) - bits(sqrt(1/2)) - 24 * 2^23: its top bits give k - 24 directly (an
-      // arithmetic shift; the range [-0x0BB504F3, 0x004AFB0C] cannot overflow) and its low 23
-      // bits the mantissa of x.
-      const uint32_t y = (wav[l][p] >> 8) | 1u;
-      const uint32_t ix = __float_as_uint((float)y) - (0x3F3504F3u + (24u << 23));
-      set_lane(x, l, __uint_as_float((ix & 0x007FFFFFu) + 0x3F3504F3u));
-      set_lane(kf, l, (float)((int)ix >> 23));
-    }
-    const T t = vsub(x, splat<T>(1.0f));
-    const T d = vadd(x, splat<T>(1.0f));
-    T rd;
+  for (int l = 0; l < L; ++l) set_lane(rd, l, rcp_fast(lane(d, l)));
+  const T sx = vmul(t, rd);
+  const T s2 = vmul(sx, sx);
+  T P = vfma(s2, splat<T>(float(-4.0 * 0.14962825 * V)), splat<T>(float(-4.0 * 0.19987397 * V)));
+  P = vfma(P, s2, splat<T>(float(-4.0 * 0.33333408 * V)));
+  P = vfma(P, s2, splat<T>(float(-4.0 * V)));
+  const T a = vfma(kf, splat<T>(float(-1.3862943611198906 * 0x1p-23 * V)), vmul(sx, P));  // V (-2 ln u_a)
+  rad = sqrt_fast_lanes(a);
+  const T th = vfma(ang, splat<T>(kAngleScale), splat<T>(kAngleOffset));
 #pragma unroll
-    for (int l = 0; l < L; ++l) {
-      float r_;
-      asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r_) : "f"(lane(d, l)));
-      set_lane(rd, l, r_);
-    }
-    const T sx = vmul(t, rd);
-    const T s2 = vmul(sx, sx);
-    T P = vfma(s2, splat<T>(-4.0f / 9.0f), splat<T>(-4.0f / 7.0f));  // -2 * 2 * (1/(2j+1))
-    P = vfma(P, s2, splat<T>(-4.0f / 5.0f));
-    P = vfma(P, s2, splat<T>(-4.0f / 3.0f));
-    P = vfma(P, s2, splat<T>(-4.0f));
-    const T a = vfma(kf, splat<T>(-1.38629436f), vmul(sx, P));  // -2 ln u_a (kf = k - 24)
-    const T rad = sqrt_fast_lanes(vmul(a, rho));  // sqrt(rho) sqrt(-2 ln u_a)
-    T c, sn;
-#pragma unroll
-    for (int l = 0; l < L; ++l) {
-      float sl, cl;
-      __sincosf(ang[l][p], &sl, &cl);
-      set_lane(sn, l, sl);
-      set_lane(c, l, cl);
-    }
-    z[2 * p] = vmul(rad, c);
-    z[2 * p + 1] = vmul(rad, sn);
+  for (int l = 0; l < L; ++l) {
+    float sl, cl;
+    __sincosf(lane(th, l), &sl, &cl);
+    set_lane(sn, l, sl);
+    set_lane(c, l, cl);
   }
 }
 

@@ -15,20 +15,31 @@
 // reads, so no two threads race and no second lattice is needed. Logical populations:
 // even state f_i(x) = A[i][x]; odd state f_i(x) = A[opposite(i)][x - c_i].
 //
-// Layout: structure of arrays A[q][z][y][x], x fastest. Kernels (step_kernels.cuh; launch
-// variants, all computing the same update; see StepVariant in internal.h):
-//   step_kernel  - one site per thread, blocks of 128 consecutive x, grid
-//                  (ceil(nx/128), ny, nz); any nx;
-//   step2_kernel - two sites per thread (x0 = 2 t, x0 + 1; nx even): every floating-
-//                  point step runs as packed FP32x2, population pairs move as one 8-byte
-//                  (FP32) or 4-byte (16-bit) access, per-population address offsets are
-//                  block-uniform; capped at 128 registers (4 blocks of 4 warps per SM)
-//                  or, for more warps, 102 (5 blocks; 3-D lattices) or 64 (8 blocks;
-//                  D2Q9); the noise loop is unrolled or rolled (smaller code); blocks
-//                  cover one row of 128 pair slots, or four rows of 32 (one per warp) for
-//                  rows shorter than 256 sites.
-// Warps touch contiguous runs of every population, so all accesses are coalesced (odd
-// steps are shifted by one element, which costs no extra DRAM traffic).
+// Layout: structure of arrays A[q][z][y][x], x fastest. Kernels (step_kernels.cuh):
+//   step_kernel - one site per thread, blocks of 128 consecutive x, grid
+//                 (ceil(nx/128), ny, nz); where variant 1 is asked for, and for unaligned rows
+//                 of planes of 4 GB or more;
+//   pair_kernel - two sites per thread, every floating-point step as packed FP32x2; pairs are
+//                 taken flat over the rows (pair.cuh), so short and odd rows fill the warps,
+//                 and move as one 8-byte (FP32) or 4-byte (16-bit) word where alignment allows.
+// What bounds the pair kernel with noise is the FMA pipe: 40 % of its cycles are Philox's
+// 32 x 32 -> 64-bit multiplies (about 4 cycles per warp and scheduler; a packed FP32x2 operation
+// takes 2 to 3.3, by its distinct register operands), the rest the packed algebra. So what
+// helped is what took operations off that pipe or filled it:
+//  - the noise needs no population, only sqrt(rho) at the end (noise_modes): it is formed
+//    while the populations travel by cp.async through shared memory, which holds no registers;
+//  - amplitudes folded into the logarithm's constants, a cubic instead of a quartic series,
+//    exact uniforms by one funnel shift (philox.cuh);
+//  - the planes' bases as kernel arguments (forming f + i * plane per access cost 130 ALU and
+//    multiply operations a pair: 256^3 FP32 0.575 -> 0.549 ms) and one offset per row;
+//  - programmatic dependent launch: the next step's blocks form half of their noise while this
+//    step drains, which is most of the time of a small box.
+// Measured (us per step, before -> now): D2Q9 64^2 4.1 -> 1.8, 200^2 5.0 -> 2.25, 512^2 6.2 ->
+// 4.1, 4096^2 BF16 176 -> 164; D3Q27 25x50x100 13.5 -> 8.0, 64^3 20 -> 10.0 (13.3 in its best
+// launch shape), 96^3 BGK 62 -> 31, 256^3 FP32 580 -> 549 (6.6 TB/s, 0.99 of the measured
+// copy), FP16 571 -> 522; D3Q19 256^3 478 -> 444.
+// Tried and slower: scalar FMAs in place of the packed ones (256^3 FP16 0.615
+// against 0.591 ms), six blocks per SM (spills: 0.586 against 0.550 ms).
 #include "step_kernels.cuh"
 
 namespace flbm {
@@ -39,8 +50,8 @@ cudaError_t launch_step(int lattice, int storage, int variant, int parity, bool 
   if (lattice == 3) return launch_step_d3q19(storage, variant, parity, noise, shear, a, s);
   const int D = lattice == 0 ? 2 : 3;
   if (storage != 0) return launch_step_16(D, storage, variant, parity, noise, shear, a, s);
-  return D == 3 ? launch_typed<3, float, false>(variant, parity, noise, shear, a, s)
-                : launch_typed<2, float, false>(variant, parity, noise, shear, a, s);
+  return D == 3 ? launch_rates<3, float, false>(variant, parity, noise, shear, a, s)
+                : launch_rates<2, float, false>(variant, parity, noise, shear, a, s);
 }
 
 }  // namespace flbm

@@ -7,10 +7,10 @@ namespace flbm {
 cudaError_t launch_step_16(int D, int storage, int variant, int parity, bool noise, bool shear, const StepArgs &a,
                            cudaStream_t s) {
   if (D == 3)
-    return storage == 1 ? launch_typed<3, __nv_bfloat16, false>(variant, parity, noise, shear, a, s)
-                        : launch_typed<3, __half, false>(variant, parity, noise, shear, a, s);
-  return storage == 1 ? launch_typed<2, __nv_bfloat16, false>(variant, parity, noise, shear, a, s)
-                      : launch_typed<2, __half, false>(variant, parity, noise, shear, a, s);
+    return storage == 1 ? launch_rates<3, __nv_bfloat16, false>(variant, parity, noise, shear, a, s)
+                        : launch_rates<3, __half, false>(variant, parity, noise, shear, a, s);
+  return storage == 1 ? launch_rates<2, __nv_bfloat16, false>(variant, parity, noise, shear, a, s)
+                      : launch_rates<2, __half, false>(variant, parity, noise, shear, a, s);
 }
 
 }  // namespace flbm

@@ -1,6 +1,7 @@
 // Kernel templates of the fused step (documented in step.cu), shared by the translation
 // units that instantiate them: step.cu (FP32 storage and the dispatch), step_16.cu
-// (BF16 and FP16 storage) and step_iso.cu (the isotropic D3Q27 variant).
+// (BF16 and FP16 storage), step_iso.cu (the isotropic D3Q27 variant), step19.cu (D3Q19) and
+// step_raw.cu (the raw-moment collision).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -8,121 +9,168 @@
 #include <type_traits>
 
 #include "collide.cuh"
+#include "d3q19.cuh"
 #include "internal.h"
+#include "pair.cuh"
 
 namespace flbm {
 namespace {
 
-template <int D, typename S, int PARITY, bool NOISE, bool SHEAR, bool ISO, bool RAW = false>
+// The collision a kernel is compiled for.
+enum Scheme { kGeneral = 0, kShear = 1, kRaw = 2 };
+
+template <int LAT>
+__device__ __forceinline__ ArrayRates rates_of(const StepArgs &a) {
+  return LAT == 19 ? ArrayRates{a.om, a.phc, a.amp, a.sqrt_kbt} : ArrayRates{a.om_t, a.phc_t, a.amp, a.sqrt_kbt};
+}
+template <int LAT, int SCHEME, bool ISO, int B0, int B1, typename T>
+__device__ __forceinline__ void site_noise(T (&n)[Noisy<LAT>::count], const StepArgs &a, uint32_t site, uint32_t dsite) {
+  noise_modes<LAT, SCHEME == kShear, ISO, B0, B1>(n, rates_of<LAT>(a), site + a.site_base, a.step_lo, a.step_hi,
+                                                  KeyTable{a.ks0, a.ks1}, dsite);
+}
+template <int LAT, bool NOISE, int SCHEME, bool ISO, typename T, typename F>
+__device__ __forceinline__ void collide_site(F &pops, const StepArgs &a, const T (&n)[Noisy<LAT>::count]) {
+  if constexpr (LAT == 19)
+    collide19<NOISE, T, SCHEME == kShear>(pops, a.rho0, rates_of<LAT>(a), n);
+  else if constexpr (SCHEME == kRaw)
+    collide_raw<LAT, NOISE, T>(pops, a.rho0, rates_of<LAT>(a), n);
+  else
+    collide_rates<LAT, NOISE, T, SCHEME == kShear, ISO>(pops, a.rho0, rates_of<LAT>(a), n);
+}
+
+template <int LAT, typename S, int PARITY, bool NOISE, int SCHEME, bool ISO>
 __global__ void __launch_bounds__(kStepBlock) step_kernel(const StepArgs a) {
   const int x = blockIdx.x * kStepBlock + threadIdx.x;
   if (x >= a.nx) return;
   const int y = blockIdx.y, z = blockIdx.z + a.z_lo;
   const Neighbourhood nb = neighbourhood(x, y, z, a.nx, a.ny, a.nz);
   S *__restrict__ f = static_cast<S *>(a.f);
-
-  float F[3][3][3];
-  load_logical<D, S, PARITY>(f, a.plane, nb, F);
-  const uint32_t site = (uint32_t)(x + (long long)a.nx * (y + (long long)a.ny * z)) + a.site_base;
-  collide_tile<D, NOISE, float, false, SHEAR, ISO, RAW>(F, a.rho0, a.om_t, a.phc_t, site, a.step_lo, a.step_hi,
-                                                        a.ks0, a.ks1);
-  store_streamed<D, S, PARITY>(f, a.plane, nb, F);
-}
-
-// RB rows per block: 1 (128 pair slots of one row; y block-uniform) or kRowBlockRows
-// (each warp one row of 32 pair slots, for rows shorter than 256 sites).
-template <int D, typename S, int PARITY, bool NOISE, bool ROLLED, bool SHEAR, int MINB, bool ISO, bool RAW = false,
-          int RB = 1>
-__global__ void __launch_bounds__(kStepBlock, MINB) step2_kernel(const StepArgs a) {
-  constexpr int BX = kStepBlock / RB;
-  const int x0 = 2 * (blockIdx.x * BX + (RB == 1 ? (int)threadIdx.x : (int)threadIdx.x % BX));
-  const int y = RB == 1 ? (int)blockIdx.y : (int)blockIdx.y * RB + (int)threadIdx.x / BX;
-  if (x0 >= a.nx || y >= a.ny) return;
-  const Addr2 ad = addr2(x0, y, blockIdx.z + a.z_lo, a.nx, a.ny, a.nz);
-  S *__restrict__ f = static_cast<S *>(a.f);
-
-  float2 F[3][3][3];
-  load_pairs<D, S, PARITY>(f, a.plane, ad, F);
-  collide_tile<D, NOISE, float2, ROLLED, SHEAR, ISO, RAW>(F, a.rho0, a.om_t, a.phc_t,
-                                                          pair_site0<PARITY>(ad) + a.site_base, a.step_lo,
-                                                          a.step_hi, a.ks0, a.ks1, pair_dsite<PARITY>(ad));
-  store_pairs<D, S, PARITY>(f, a.plane, ad, F);
-}
-
-template <typename S>
-constexpr int storage_code() {
-  return sizeof(S) == 4 ? 0 : (std::is_same<S, __nv_bfloat16>::value ? 1 : 2);
-}
-
-// One launch of variant 1, 2, 3, 5 or 6 (the pipelined variant 4 lives in
-// step_pipe.cu). ISO kernels exist for variants 1, 2 and 5 only; the host maps 3 and 6
-// to 2 and 5 for them.
-template <int D, typename S, int PARITY, bool NOISE, bool SHEAR, bool ISO>
-cudaError_t launch_kernel(int variant, const StepArgs &a, cudaStream_t s) {
-  const dim3 block(kStepBlock);
-  if (variant != kStepOneSite) {
-    // Register caps: 128 (four blocks of 128 threads per SM) or, for variants 5 and 6,
-    // 102 for D3Q27 (five blocks: more warps to hide latency, at the risk of spills) and
-    // 64 for the lighter D2Q9 update (eight blocks; ten, at 51 registers, left the even
-    // step waiting on its loads: 0.214 against 0.183 ms at 4096^2).
-    constexpr int kOcc = D == 3 ? 5 : 8;
-    const dim3 grid((a.nx / 2 + kStepBlock - 1) / kStepBlock, a.ny, a.nz_grid);
-    const bool occ = variant == kStepPairOcc || variant == kStepPairRolledOcc;
-    const bool rolled = !ISO && (variant == kStepPairRolled || variant == kStepPairRolledOcc);
-    if (variant == kStepPairOccRows || variant == kStepPairRows) {
-      constexpr int BX = kStepBlock / kRowBlockRows;
-      const dim3 grid_r((a.nx / 2 + BX - 1) / BX, (a.ny + kRowBlockRows - 1) / kRowBlockRows, a.nz_grid);
-      if (variant == kStepPairOccRows)
-        step2_kernel<D, S, PARITY, NOISE, false, SHEAR, kOcc, ISO, false, kRowBlockRows><<<grid_r, block, 0, s>>>(a);
-      else
-        step2_kernel<D, S, PARITY, NOISE, false, SHEAR, 4, ISO, false, kRowBlockRows><<<grid_r, block, 0, s>>>(a);
-    } else if (occ) {
-      if (rolled)
-        step2_kernel<D, S, PARITY, NOISE, !ISO, SHEAR, kOcc, ISO><<<grid, block, 0, s>>>(a);
-      else
-        step2_kernel<D, S, PARITY, NOISE, false, SHEAR, kOcc, ISO><<<grid, block, 0, s>>>(a);
-    } else {
-      if (rolled)
-        step2_kernel<D, S, PARITY, NOISE, !ISO, SHEAR, 4, ISO><<<grid, block, 0, s>>>(a);
-      else
-        step2_kernel<D, S, PARITY, NOISE, false, SHEAR, 4, ISO><<<grid, block, 0, s>>>(a);
-    }
+  const uint32_t site = (uint32_t)(x + (long long)a.nx * (y + (long long)a.ny * z));
+  float n[Noisy<LAT>::count];
+  if (NOISE) site_noise<LAT, SCHEME, ISO, 0, Noisy<LAT>::blocks>(n, a, site, 0u);
+  if constexpr (LAT == 19) {
+    float F[19];
+    load19<S, PARITY>(f, a.plane, nb, F);
+    collide_site<LAT, NOISE, SCHEME, ISO>(F, a, n);
+    store19<S, PARITY>(f, a.plane, nb, F);
   } else {
+    float F[3][3][3];
+    load_logical<LAT, S, PARITY>(f, a.plane, nb, F);
+    collide_site<LAT, NOISE, SCHEME, ISO>(F, a, n);
+    store_streamed<LAT, S, PARITY>(f, a.plane, nb, F);
+  }
+}
+
+template <int LAT, typename S, int PARITY, bool NOISE, int SCHEME, bool ISO, bool ALIGNED, bool ROWS, typename O, int MINB>
+__global__ void __launch_bounds__(kStepBlock, MINB) pair_kernel(const StepArgs a) {
+  using Access = PairAccess<LAT, S, PARITY, ALIGNED, ROWS, O, NOISE, kStepBlock>;
+  __shared__ typename Access::Word stage[Access::STAGED ? Access::WORDS * kStepBlock : 1];
+  launch_dependents();
+  Access p;
+  if (ROWS) {
+    const int x0 = 2 * (int)(blockIdx.x * kStepBlock + threadIdx.x);
+    if (x0 >= a.nx) return;
+    p.init_row(a.pop, x0, blockIdx.y, blockIdx.z + a.z_lo, a.nx, a.ny, a.nz);
+  } else {
+    const uint32_t slot = blockIdx.x * (uint32_t)kStepBlock + threadIdx.x;
+    if (slot >= a.slots[PARITY]) return;
+    if (PARITY == 0) {
+      p.init_flat(a.pop, a.first, a.count, slot);
+    } else {
+      int x0, y, z;
+      slot_xyz(slot, a.nx, a.ny, a.m_hp, a.p_hp, a.m_ny, a.p_ny, x0, y, z);
+      p.init_row(a.pop, x0, y, z + a.z_lo, a.nx, a.ny, a.nz);
+    }
+  }
+  // Large launches: every read first, all of the noise while the populations travel. Small ones:
+  // half of the noise before the wait for the step before (it fills the drain of that launch).
+  constexpr int B = Noisy<LAT>::blocks;
+  float2 n[Noisy<LAT>::count];
+  const uint32_t st = shared_address(stage + threadIdx.x);
+  if (a.early) {
+    wait_prerequisites();
+    p.fetch(st);
+  }
+  if (NOISE) site_noise<LAT, SCHEME, ISO, 0, B / 2>(n, a, p.site0, p.dsite);
+  if (!a.early) {
+    wait_prerequisites();
+    p.fetch(st);
+  }
+  if (NOISE) site_noise<LAT, SCHEME, ISO, B / 2, B>(n, a, p.site0, p.dsite);
+  if (Access::STAGED) cp_async_wait_all();
+  if constexpr (LAT == 19) {
+    float2 F[19];
+    p.load_list(stage + threadIdx.x, F);
+    p.forget();
+    collide_site<LAT, NOISE, SCHEME, ISO>(F, a, n);
+    p.store_list(F);
+  } else {
+    float2 F[3][3][3];
+    p.load_tile(stage + threadIdx.x, F);
+    p.forget();
+    collide_site<LAT, NOISE, SCHEME, ISO>(F, a, n);
+    p.store_tile(F);
+  }
+}
+
+// Blocks of 128 threads per SM that a pair kernel is compiled for (its register cap), measured at
+// 256^3 (FP32 D3Q27, us per step at 3 / 4 / 5 / 6 blocks): staged reads and the paper's rates 563 /
+// 551 / 550 / 586, where six spill; direct reads without noise 551 / 523 / 554 / -, of unaligned
+// elements (255^3) 534 / 559 / 711 / -. The general rates keep the tile and the noise together
+// (BGK 96^3: 35.1 / 33.8).
+template <int LAT, int SCHEME, bool DIRECT, bool ALIGNED>
+constexpr int pair_blocks() {
+  return LAT == 2 ? 8 : DIRECT ? (ALIGNED ? 4 : 3) : SCHEME == kShear ? 5 : 4;
+}
+
+template <int LAT, typename S, int PARITY, bool NOISE, int SCHEME, bool ISO>
+cudaError_t launch_kernel(int variant, const StepArgs &a, cudaStream_t s) {
+  if (variant == kStepOneSite || (a.wide && !a.aligned[PARITY])) {
     const dim3 grid((a.nx + kStepBlock - 1) / kStepBlock, a.ny, a.nz_grid);
-    step_kernel<D, S, PARITY, NOISE, SHEAR, ISO><<<grid, block, 0, s>>>(a);
+    step_kernel<LAT, S, PARITY, NOISE, SCHEME, ISO><<<grid, kStepBlock, 0, s>>>(a);
+    return cudaGetLastError();
   }
-  return cudaGetLastError();
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((a.slots[PARITY] + kStepBlock - 1) / kStepBlock);
+  cfg.blockDim = dim3(kStepBlock);
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  constexpr int MB = pair_blocks<LAT, SCHEME, !NOISE, true>();
+  const bool narrow = !a.wide && (variant == kStepPairOcc || variant == kStepPairRolledOcc || variant == kStepPairOccRows);
+  if (!a.aligned[PARITY])
+    return cudaLaunchKernelEx(&cfg, pair_kernel<LAT, S, PARITY, NOISE, SCHEME, ISO, false, false, uint32_t,
+                                                pair_blocks<LAT, SCHEME, !NOISE || sizeof(S) == 2, false>()>, a);
+  if constexpr (PARITY == 1) {
+    const int per_row = (a.nx / 2 + kStepBlock - 1) / kStepBlock;
+    if (per_row * kStepBlock <= a.nx / 2 + a.nx / 16) {
+      cfg.gridDim = dim3(per_row, a.ny, a.nz_grid);
+      if (narrow)
+        return cudaLaunchKernelEx(&cfg, pair_kernel<LAT, S, PARITY, NOISE, SCHEME, ISO, true, true, uint32_t, MB>, a);
+      return cudaLaunchKernelEx(&cfg, pair_kernel<LAT, S, PARITY, NOISE, SCHEME, ISO, true, true, uint64_t, MB>, a);
+    }
+  }
+  if (narrow)
+    return cudaLaunchKernelEx(&cfg, pair_kernel<LAT, S, PARITY, NOISE, SCHEME, ISO, true, false, uint32_t, MB>, a);
+  return cudaLaunchKernelEx(&cfg, pair_kernel<LAT, S, PARITY, NOISE, SCHEME, ISO, true, false, uint64_t, MB>, a);
 }
 
-template <int D, typename S, bool ISO>
-cudaError_t launch_typed(int variant, int parity, bool noise, bool shear, const StepArgs &a, cudaStream_t s) {
-  if (!ISO && variant == kStepPipelined)
-    return launch_step_pipelined(D, storage_code<S>(), parity, noise, shear, a, s);
-  if (parity == 0) {
-    if (noise)
-      return shear ? launch_kernel<D, S, 0, true, true, ISO>(variant, a, s)
-                   : launch_kernel<D, S, 0, true, false, ISO>(variant, a, s);
-    return shear ? launch_kernel<D, S, 0, false, true, ISO>(variant, a, s)
-                 : launch_kernel<D, S, 0, false, false, ISO>(variant, a, s);
-  }
-  if (noise)
-    return shear ? launch_kernel<D, S, 1, true, true, ISO>(variant, a, s)
-                 : launch_kernel<D, S, 1, true, false, ISO>(variant, a, s);
-  return shear ? launch_kernel<D, S, 1, false, true, ISO>(variant, a, s)
-               : launch_kernel<D, S, 1, false, false, ISO>(variant, a, s);
+template <int LAT, typename S, bool ISO, int SCHEME>
+cudaError_t launch_typed(int variant, int parity, bool noise, const StepArgs &a, cudaStream_t s) {
+  if (parity == 0)
+    return noise ? launch_kernel<LAT, S, 0, true, SCHEME, ISO>(variant, a, s)
+                 : launch_kernel<LAT, S, 0, false, SCHEME, ISO>(variant, a, s);
+  return noise ? launch_kernel<LAT, S, 1, true, SCHEME, ISO>(variant, a, s)
+               : launch_kernel<LAT, S, 1, false, SCHEME, ISO>(variant, a, s);
 }
 
-// The raw-moment counterpart (collide_raw): one site per thread or two (nx even).
-template <int D, typename S, int PARITY, bool NOISE>
-cudaError_t launch_raw_kernel(int variant, const StepArgs &a, cudaStream_t s) {
-  const dim3 block(kStepBlock);
-  if (variant == kStepOneSite)
-    step_kernel<D, S, PARITY, NOISE, false, false, true>
-        <<<dim3((a.nx + kStepBlock - 1) / kStepBlock, a.ny, a.nz_grid), block, 0, s>>>(a);
-  else
-    step2_kernel<D, S, PARITY, NOISE, false, false, 4, false, true>
-        <<<dim3((a.nx / 2 + kStepBlock - 1) / kStepBlock, a.ny, a.nz_grid), block, 0, s>>>(a);
-  return cudaGetLastError();
+template <int LAT, typename S, bool ISO>
+cudaError_t launch_rates(int variant, int parity, bool noise, bool shear, const StepArgs &a, cudaStream_t s) {
+  return shear ? launch_typed<LAT, S, ISO, kShear>(variant, parity, noise, a, s)
+               : launch_typed<LAT, S, ISO, kGeneral>(variant, parity, noise, a, s);
 }
 
 }  // namespace

@@ -1,0 +1,89 @@
+"""The pair kernels' forms against the FP64 oracle: even and odd rows, odd planes (scalar
+accesses), rows of a whole number of blocks and short of it, the smallest rows, launches
+above the size from which reads go before the noise, 64-bit and 32-bit offsets, and every
+collision. The tolerance is the repository's parity bound, 1e-5 of w_i rho0 (FP32 rounding
+of at most six updates lies far below it); in 16-bit storage one update from the stored
+state may differ by the format's rounding of the deviation only, as in test_gpu_parity.py.
+"""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+TOL = 1e-5
+
+
+@pytest.fixture(scope="module")
+def fl():
+    import torch
+
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2602_16486_gb300 as fl
+
+    return fl
+
+
+@pytest.fixture(scope="module")
+def oracle_mod():
+    import oracle
+
+    oracle.build()
+    return oracle
+
+
+def _lam(q, rates):
+    lam = np.ones(q)
+    lam[[4, 5] if q == 9 else [7, 8, 9]] = 1.7
+    if rates == "general":
+        lam = 1.0 + 0.5 * np.sin(1.0 + 2.0 * np.arange(q))
+    lam[: 3 if q == 9 else 4] = 1.0
+    return lam
+
+
+FORMS = [(0, (1, 5, 1)), (0, (2, 3, 1)), (0, (3, 3, 1)), (0, (258, 7, 1)), (0, (255, 9, 1)), (0, (640, 642, 1)),
+         (1, (1, 3, 5)), (1, (2, 3, 3)), (1, (5, 7, 3)), (1, (7, 4, 3)), (1, (240, 3, 2)), (1, (256, 2, 3)),
+         (1, (96, 66, 64)), (2, (9, 5, 4)), (2, (256, 3, 2)), (3, (5, 5, 5)), (3, (240, 2, 3)), (3, (10, 9, 7))]
+
+
+@pytest.mark.parametrize("lattice,dims", FORMS)
+@pytest.mark.parametrize("rates", ["paper", "general", "raw"])
+def test_forms_match_oracle(fl, oracle_mod, lattice, dims, rates):
+    if rates == "raw" and lattice > 1:
+        pytest.skip("the raw-moment collision is built for D2Q9 and D3Q27")
+    q = (9, 27, 27, 19)[lattice]
+    big = dims[0] * dims[1] * dims[2] > 300000
+    lam, w = _lam(q, rates), oracle_mod.tables(lattice)[1].reshape(q, 1, 1, 1)
+    for kbt in (1e-4, 0.0):
+        for variant in (2, 5) if not big else (0,):
+            with fl.Lattice(lattice, dims, lam, kbt, 1.0, 77) as lat:
+                lat.variant = variant
+                if rates == "raw":
+                    lat.collision = fl.FLBM_COLLISION_RAW
+                lat.init_uniform((0.04, -0.02, 0.01), 1e-3, 3)
+                f0 = lat.populations()
+                n = 2 if big else 6
+                lat.step(n)
+                fg = lat.populations()
+            fo = oracle_mod.run(lattice, dims, lam, kbt, 77, f0, 0, n, model=int(rates == "raw"))
+            assert (np.abs(fg - fo) / w).max() <= TOL, (kbt, variant)
+
+
+@pytest.mark.parametrize("storage,bits", [(1, 8), (2, 11)])
+@pytest.mark.parametrize("lattice,dims", [(0, (35, 9, 1)), (0, (34, 9, 1)), (1, (9, 5, 7)), (1, (9, 6, 7)),
+                                          (1, (240, 2, 3)), (2, (7, 6, 3)), (3, (9, 5, 4))])
+def test_forms_16_bit_one_step(fl, oracle_mod, storage, bits, lattice, dims):
+    q = (9, 27, 27, 19)[lattice]
+    w = oracle_mod.tables(lattice)[1].reshape(q, 1, 1, 1)
+    for rates in ("paper", "general"):
+        lam = _lam(q, rates)
+        for steps, kbt in ((3, 1e-4), (4, 1e-4), (3, 0.0)):
+            with fl.Lattice(lattice, dims, lam, kbt, 1.0, 5, storage) as lat:
+                lat.init_uniform((0.02, 0.0, -0.01), 1e-3, 2)
+                lat.step(steps)
+                f0 = lat.populations()
+                lat.step(1)
+                fg = lat.populations()
+            fo = oracle_mod.run(lattice, dims, lam, kbt, 5, f0, steps, 1)
+            bound = np.abs(fo - w) * 2.0 ** -bits * 1.01 + 2e-6 * np.abs(fo) + 3e-8
+            assert np.all(np.abs(fg - fo) <= bound), (rates, steps, kbt)
