@@ -985,8 +985,13 @@ int batch_shape(flbm_batch *b) {
     if (total > 0x3fffffffLL) return fail(FLBM_EINVAL, "too many tiles");
   }
   if (n3 == nl) tiles3 = total;
-  b->g3 = BatchGroup{0, n3, 0, int(tiles3)};
-  b->g2 = BatchGroup{n3, nl, int(tiles3), int(total - tiles3)};
+  const auto wide = [&](int lo, int hi) {
+    bool w = false;
+    for (int i = lo; i < hi; ++i) w = w || b->members[size_t(b->order[size_t(i)])]->f_bytes > 0xFFFFFFFFull;
+    return w;
+  };
+  b->g3 = BatchGroup{0, n3, 0, int(tiles3), wide(0, n3)};
+  b->g2 = BatchGroup{n3, nl, int(tiles3), int(total - tiles3), wide(n3, nl)};
   FLBM_CUDA(cudaStreamSynchronize(b->stream));
   batch_drop_graphs(b);
   b->tiles_for = 0;

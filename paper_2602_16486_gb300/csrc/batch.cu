@@ -4,12 +4,18 @@
 // with its own parameters.
 //
 // The host lays every lattice's populations out in one allocation and cuts all lattices
-// into tiles of equal pair-slot count (one slot of two x-adjacent sites per thread; a
+// into tiles of equal pair-slot count (one slot of two sites per thread, pair.cuh; a
 // tile may span rows, never lattices). Two launch structures (BatchForm):
 //
 // Per-step forms (the default): per step one plain launch per lattice type, block b on
 // tile tile0 + b, the hardware block scheduler balancing the load; the n launches of a
-// call are captured once into a CUDA graph and replayed.
+// call are captured once into a CUDA graph and replayed. The kernel is the single lattice's
+// (pair_kernel, step_kernels.cuh): reads staged by cp.async while the noise is formed, the next
+// launch's blocks starting as this one drains. It is bound like it by the FMA pipe; what a batch
+// adds is the addressing (a lattice's array and plane are not kernel arguments of their own).
+// us per step, before -> now, in the shape the autotuner picks: 32 D3Q27 64^3 321 -> 281, one
+// 256^3 634 -> 568, 233 of 33^3 368 -> 338, 512 of 16^3 86 -> 74, 256 D2Q9 256^2 201 -> 195, 256 of
+// 255^2 228 -> 216; 256 mixed lattices (10.7 M sites) 392 -> 360.
 //
 // Persistent form: one cooperative launch runs n steps; block b takes the work items
 // (step s, tile b + j G) in step-major order. There is no grid-wide barrier between
@@ -41,188 +47,108 @@ namespace flbm {
 namespace {
 
 
-// The collision with lattice L's parameters: its three shear-structure numbers (SHEAR:
-// per-mode factors are compile-time constants) or its per-mode arrays; round keys are
-// formed from its key.
-template <int D, bool SHEAR, bool ROLLED>
-__device__ __forceinline__ void collide_lattice(float2 (&F)[3][3][3], const BatchLattice &L, const float *rates,
-                                                uint32_t s0, uint32_t dsite, uint32_t step_lo, uint32_t step_hi) {
-  const KeyBase keys{L.key0, L.key1};
-  float2 n[Noisy<D>::count];
-  if (SHEAR) {
-    const ShearRates<D> r{L.sqrt_kbt, L.om_shear, L.amp_shear};
-    noise_modes<D, true, false, 0, Noisy<D>::blocks>(n, r, s0, step_lo, step_hi, keys, dsite);
-    collide_rates<D, true, float2, true>(F, L.rho0, r, n);
-  } else {
-    const ArrayRates r{rates, rates + 27, nullptr, 0.0f};
-    noise_modes<D, false, false, 0, Noisy<D>::blocks>(n, r, s0, step_lo, step_hi, keys, dsite);
-    collide_rates<D, true, float2, false>(F, L.rho0, r, n);
-  }
-}
-
-// Pair slots of lattice L: row r = y + ny z holds ceil(nx / 2) slots, and slot j of it
-// is the sites x0 = 2 j and x0 + 1 (only x0 in the last slot of a row when nx is odd).
-// Slots are numbered row-major, so consecutive slots are consecutive sites and a warp's
-// accesses stay contiguous for every nx.
+// The pair slots of lattice L (pair.cuh): rows of ceil(nx / 2) slots, numbered row-major, so a
+// tile spans rows and a warp's accesses stay contiguous for every nx. From an even step count
+// slot k is the flat sites 2k and 2k + 1 instead, and the last slots of odd rows stay empty.
 __device__ __forceinline__ uint32_t pair_slots(const BatchLattice &L) {
   return (uint32_t)((L.nx + 1) >> 1) * (uint32_t)L.ny * (uint32_t)L.nz;
 }
-
-// Row coordinates of pair slot `slot` (32-bit arithmetic: every site index is < 2^32, so
-// slots and rows are < 2^31) and the site index of its first site: 2 slot when nx is even,
-// 2 slot - r otherwise. The divisions use the lattice's multiply-shift constants.
-__device__ __forceinline__ uint32_t slot_xyz(const BatchLattice &L, uint32_t slot, int &x0, int &y, int &z) {
-  const uint32_t hp = (uint32_t)((L.nx + 1) >> 1);
-  const uint32_t r = udiv_magic(slot, L.m_hp, L.p_hp());
-  x0 = 2 * (int)(slot - r * hp);
-  const uint32_t q = udiv_magic(r, L.m_ny, L.p_ny());
-  y = (int)(r - q * (uint32_t)L.ny);
-  z = (int)q;
-  return 2u * slot - ((L.nx & 1) ? r : 0u);
+template <int PARITY>
+__device__ __forceinline__ bool pairs_aligned(const BatchLattice &L) {
+  return PARITY == 0 ? (L.plane & 1u) == 0u : (L.nx & 1) == 0;
 }
 
-// Sites of a pair slot of an odd-nx row: x0 - 1, x0, x0 + 1 and x0 + 2 (periodic), and
-// the periodic row / plane offsets as in Addr2. Lane 0 is site x0 and uses s[0..2]; lane
-// 1 is x0 + 1 and uses s[1..3]. In the last slot of a row (x0 = nx - 1) lane 1 wraps to
-// a real site of the same row: it is loaded and collided (every access stays inside the
-// lattice) but never stored.
-struct OddPair {
-  long long s[4];
-  long long dy[3], dz[3];
-};
-
-__device__ __forceinline__ OddPair odd_pair(int x0, int y, int z, int nx, int ny, int nz) {
-  OddPair a;
-  const long long row = ((long long)z * ny + y) * nx;
-  int x1 = x0 + 1;
-  if (x1 >= nx) x1 -= nx;
-  int x2 = x1 + 1;
-  if (x2 >= nx) x2 -= nx;
-  a.s[0] = row + (x0 == 0 ? nx - 1 : x0 - 1);
-  a.s[1] = row + x0;
-  a.s[2] = row + x1;
-  a.s[3] = row + x2;
-  const long long rl = nx, pl = (long long)nx * ny;
-  a.dy[0] = (y == 0) ? (long long)(ny - 1) * rl : -rl;
-  a.dy[1] = 0;
-  a.dy[2] = (y == ny - 1) ? -(long long)(ny - 1) * rl : rl;
-  a.dz[0] = (z == 0) ? (long long)(nz - 1) * pl : -pl;
-  a.dz[1] = 0;
-  a.dz[2] = (z == nz - 1) ? -(long long)(nz - 1) * pl : pl;
-  return a;
-}
-
-// As load_logical2 for an odd-nx pair: scalar accesses (the pair is not 8-byte aligned).
-template <int D, int PARITY>
-__device__ __forceinline__ void load_odd_pair(const float *__restrict__ f, long long plane, const OddPair &ad,
-                                              float2 (&F)[3][3][3]) {
-  constexpr int z0 = (D == 3) ? -1 : 0, z1 = (D == 3) ? 1 : 0;
-#pragma unroll
-  for (int dz = z0; dz <= z1; ++dz)
-#pragma unroll
-    for (int dy = -1; dy <= 1; ++dy)
-#pragma unroll
-      for (int dx = -1; dx <= 1; ++dx) {
-        const int i = Lat<D>::index(dx, dy, dz);
-        float2 v;
-        if (PARITY == 0) {
-          const float *b = f + i * plane;
-          v.x = b[ad.s[1]];
-          v.y = b[ad.s[2]];
-        } else {
-          // f_i(x) = A[opposite(i)][x - c_i]
-          const float *b = f + opposite<D>(i) * plane + ad.dy[1 - dy] + ad.dz[1 - dz];
-          v.x = b[ad.s[1 - dx]];
-          v.y = b[ad.s[2 - dx]];
-        }
-        F[dz + 1][dy + 1][dx + 1] = v;
-      }
-}
-
-// As store_streamed2 for an odd-nx pair; lane 1 only when `two`.
-template <int D, int PARITY>
-__device__ __forceinline__ void store_odd_pair(float *__restrict__ f, long long plane, const OddPair &ad, bool two,
-                                               const float2 (&F)[3][3][3]) {
-  constexpr int z0 = (D == 3) ? -1 : 0, z1 = (D == 3) ? 1 : 0;
-#pragma unroll
-  for (int dz = z0; dz <= z1; ++dz)
-#pragma unroll
-    for (int dy = -1; dy <= 1; ++dy)
-#pragma unroll
-      for (int dx = -1; dx <= 1; ++dx) {
-        const int i = Lat<D>::index(dx, dy, dz);
-        const float2 v = F[dz + 1][dy + 1][dx + 1];
-        float *b;
-        int k0, k1;
-        if (PARITY == 0) {
-          b = f + opposite<D>(i) * plane;
-          k0 = 1;
-          k1 = 2;
-        } else {
-          // f*_i(x) goes to A[i][x + c_i]
-          b = f + i * plane + ad.dy[1 + dy] + ad.dz[1 + dz];
-          k0 = 1 + dx;
-          k1 = 2 + dx;
-        }
-        b[ad.s[k0]] = v.x;
-        if (two) b[ad.s[k1]] = v.y;
-      }
-}
-
-// The two sites of pair slot `slot` of lattice L. EVEN (nx even): the sites share a row
-// and move as 8-byte pairs (Addr2, as the single-lattice kernels). Otherwise scalar
-// accesses through OddPair. Either way the neighbour addresses are recomputed at the
-// store rather than kept live across the collision (register pressure).
-template <int D, int PARITY, bool SHEAR, bool EVEN, bool ROLLED = true>
-__device__ __forceinline__ void batch_sites(const BatchLattice &L, char *pool, const float *rates, uint32_t slot,
-                                            uint32_t step_lo, uint32_t step_hi) {
-  float *__restrict__ f = reinterpret_cast<float *>(pool + 256ull * L.f256);
-  const long long plane = L.plane;
-  float2 F[3][3][3];
-  uint32_t s0, dsite = 1u;
-  {
+// The pair of slot `slot` of lattice L.
+template <int D, int PARITY, bool ALIGNED, bool STAGE, typename O, int THREADS, typename Base>
+__device__ __forceinline__ auto pair_of(const BatchLattice &L, const Base &planes, uint32_t slot) {
+  PairAccess<D, float, PARITY, ALIGNED, false, O, STAGE, THREADS, Base> p;
+  if (PARITY == 0) {
+    p.init_flat(planes, 0u, L.plane, slot);
+  } else {
     int x0, y, z;
-    s0 = slot_xyz(L, slot, x0, y, z);
-    if (EVEN) {  // the single-lattice pairing: odd steps take sites x0 + 1 and x0 + 2
-      const Addr2 ad = addr2(x0, y, z, L.nx, L.ny, L.nz);
-      load_pairs<D, float, PARITY>(f, plane, ad, F);
-      s0 = pair_site0<PARITY>(ad);
-      dsite = pair_dsite<PARITY>(ad);
-    } else {
-      load_odd_pair<D, PARITY>(f, plane, odd_pair(x0, y, z, L.nx, L.ny, L.nz), F);
-    }
+    slot_xyz(slot, L.nx, L.ny, L.m_hp, L.p_hp(), L.m_ny, L.p_ny(), x0, y, z);
+    p.init_row(planes, x0, y, z, L.nx, L.ny, L.nz);
   }
-  collide_lattice<D, SHEAR, ROLLED>(F, L, rates, s0, dsite, step_lo, step_hi);
-  // The empty asm hides the slot's provenance so that the compiler cannot merge the
-  // store's address computation with the load's (and keep 18 registers live).
+  return p;
+}
+
+// The noise and the collision with lattice L's parameters: its three shear-structure numbers
+// (SHEAR) or its per-mode arrays; round keys are formed from its key.
+template <int D, bool SHEAR, int B0, int B1>
+__device__ __forceinline__ void lattice_noise(float2 (&n)[Noisy<D>::count], const BatchLattice &L, const float *rates,
+                                              uint32_t s0, uint32_t dsite, unsigned long long step) {
+  const KeyBase keys{L.key0, L.key1};
+  const uint32_t lo = (uint32_t)step, hi = (uint32_t)(step >> 32);
+  if (SHEAR)
+    noise_modes<D, true, false, B0, B1>(n, ShearRates<D>{L.sqrt_kbt, L.om_shear, L.amp_shear}, s0, lo, hi, keys, dsite);
+  else
+    noise_modes<D, false, false, B0, B1>(n, ArrayRates{rates, rates + 27, nullptr, 0.0f}, s0, lo, hi, keys, dsite);
+}
+template <int D, bool SHEAR>
+__device__ __forceinline__ void lattice_collide(float2 (&F)[3][3][3], const BatchLattice &L, const float *rates,
+                                                const float2 (&n)[Noisy<D>::count]) {
+  if (SHEAR)
+    collide_rates<D, true, float2, true>(F, L.rho0, ShearRates<D>{L.sqrt_kbt, L.om_shear, L.amp_shear}, n);
+  else
+    collide_rates<D, true, float2, false>(F, L.rho0, ArrayRates{rates, rates + 27, nullptr, 0.0f}, n);
+}
+
+// One pair of lattice L in a per-step launch: as pair_kernel (step_kernels.cuh), `early` likewise.
+// Only the reads and writes are compiled for both alignments; `stage` (STAGE) holds the pair in
+// the same layout for both.
+template <int D, int PARITY, bool SHEAR, typename O, bool STAGE, int THREADS, typename Base>
+__device__ __forceinline__ void batch_pair(const BatchLattice &L, const Base &planes, const float *rates, uint32_t slot,
+                                           unsigned long long step, bool early, float2 *stage) {
+  const bool aligned = pairs_aligned<PARITY>(L);
+  if (PARITY == 0 && 2ull * slot >= L.plane) return;
+  constexpr int B = Noisy<D>::blocks;
+  float2 n[Noisy<D>::count], F[3][3][3];
+  uint32_t s0, dsite;
+  const auto begin = [&](bool read) {
+    if (read) wait_prerequisites();
+    if (aligned) {
+      const auto p = pair_of<D, PARITY, true, STAGE, O, THREADS>(L, planes, slot);
+      s0 = p.site0;
+      dsite = p.dsite;
+      if (read && STAGE) p.fetch(shared_address(stage));
+    } else {
+      const auto p = pair_of<D, PARITY, false, STAGE, O, THREADS>(L, planes, slot);
+      s0 = p.site0;
+      dsite = p.dsite;
+      if (read && STAGE) p.fetch(shared_address(stage));
+    }
+  };
+  begin(early);
+  lattice_noise<D, SHEAR, 0, B / 2>(n, L, rates, s0, dsite, step);
+  if (!early) begin(true);
+  lattice_noise<D, SHEAR, B / 2, B>(n, L, rates, s0, dsite, step);
+  if (STAGE) cp_async_wait_all();
+  if (STAGE || aligned)
+    pair_of<D, PARITY, true, STAGE, O, THREADS>(L, planes, slot).load_tile(stage, F);
+  else
+    pair_of<D, PARITY, false, STAGE, O, THREADS>(L, planes, slot).load_tile(stage, F);
+  lattice_collide<D, SHEAR>(F, L, rates, n);
+  // The slot is hidden so that the stores' addresses are formed anew instead of staying in
+  // registers across the collision.
   uint32_t sl = slot;
   asm volatile("" : "+r"(sl));
-  int x0, y, z;
-  slot_xyz(L, sl, x0, y, z);
-  if (EVEN)
-    store_pairs<D, float, PARITY>(f, plane, addr2(x0, y, z, L.nx, L.ny, L.nz), F);
+  if (aligned)
+    pair_of<D, PARITY, true, STAGE, O, THREADS>(L, planes, sl).store_tile(F);
   else
-    store_odd_pair<D, PARITY>(f, plane, odd_pair(x0, y, z, L.nx, L.ny, L.nz), x0 + 1 < L.nx, F);
+    pair_of<D, PARITY, false, STAGE, O, THREADS>(L, planes, sl).store_tile(F);
 }
 
-// Pair slot first + threadIdx.x of tile [first, end) of lattice L.
+// Pair slot first + threadIdx.x of tile [first, end) of lattice L (persistent form).
 template <int PARITY, bool SHEAR>
 __device__ __forceinline__ void batch_tile(const BatchLattice &L, char *pool, const float *rates, uint32_t first,
-                                           uint32_t end,
-                                           uint32_t step_lo, uint32_t step_hi) {
+                                           uint32_t end, unsigned long long step) {
   const uint32_t slot = first + threadIdx.x;
   if (slot >= end) return;
-  if (L.D() == 3) {
-    if (L.nx % 2 == 0)
-      batch_sites<3, PARITY, SHEAR, true>(L, pool, rates, slot, step_lo, step_hi);
-    else
-      batch_sites<3, PARITY, SHEAR, false>(L, pool, rates, slot, step_lo, step_hi);
-  } else {
-    if (L.nx % 2 == 0)
-      batch_sites<2, PARITY, SHEAR, true>(L, pool, rates, slot, step_lo, step_hi);
-    else
-      batch_sites<2, PARITY, SHEAR, false>(L, pool, rates, slot, step_lo, step_hi);
-  }
+  const PlaneStride planes{pool + 256ull * L.f256, 4ull * L.plane};
+  if (L.D() == 3)
+    batch_pair<3, PARITY, SHEAR, uint64_t, false, 1>(L, planes, rates, slot, step, true, nullptr);
+  else
+    batch_pair<2, PARITY, SHEAR, uint64_t, false, 1>(L, planes, rates, slot, step, true, nullptr);
 }
 
 // Thread 0: waits until lattice `lat` has finished `target` tiles in this launch.
@@ -278,11 +204,10 @@ __global__ void __launch_bounds__(kBatchMaxThreads, 2) batch_kernel(const BatchA
     const uint32_t slots = pair_slots(L);
     const uint32_t end = first + per < slots ? first + per : slots;
     const unsigned long long step = (unsigned long long)(step0 + s);
-    const uint32_t lo = (uint32_t)step, hi = (uint32_t)(step >> 32);
     if (step & 1)
-      batch_tile<1, SHEAR>(L, a.pool, a.rates + 54 * lat, first, end, lo, hi);
+      batch_tile<1, SHEAR>(L, a.pool, a.rates + 54 * lat, first, end, step);
     else
-      batch_tile<0, SHEAR>(L, a.pool, a.rates + 54 * lat, first, end, lo, hi);
+      batch_tile<0, SHEAR>(L, a.pool, a.rates + 54 * lat, first, end, step);
     __syncthreads();  // every thread's writes of this tile are issued
     if (threadIdx.x == 0) {
       __threadfence();  // release
@@ -307,10 +232,17 @@ __global__ void __launch_bounds__(kBatchMaxThreads, 2) batch_kernel(const BatchA
 // the D2Q9 blocks at the register count (and occupancy) of D2Q9 alone. The step number
 // is read from the device counter plus `k`, so that a captured graph of n such launches
 // serves every call with the same n and the same starting parity; PARITY is fixed per
-// launch.
-template <int D, bool SHEAR, int PARITY, bool ROLLED, int MINB>
-__global__ void __launch_bounds__(MINB >= 5 ? 128 : kBatchMaxThreads, MINB)
-    batch_step_kernel(const BatchArgs a, int k, int lat_lo, int lat_hi, int tile_base) {
+// launch. Every launch of a call but its first starts while the one before it drains
+// (programmatic dependent launch); the counter is only written after a call's last launch has
+// ended and before the next call's first one starts, so it may be read before the wait.
+// THREADS: 64 or 128, reads staged in shared memory, or 256, reads direct (two blocks of 256
+// stages would not fit beside each other).
+template <int D, bool SHEAR, int PARITY, typename O, int THREADS, int MINB>
+__global__ void __launch_bounds__(THREADS, MINB)
+    batch_step_kernel(const __grid_constant__ BatchArgs a, int k, int lat_lo, int lat_hi, int tile_base, bool early) {
+  constexpr bool STAGE = THREADS < 256;
+  __shared__ float2 stage[STAGE ? Lat<D>::Q * THREADS : 1];
+  launch_dependents();
   const int t = tile_base + (int)blockIdx.x;
   const int lat = lattice_of(a, t, lat_lo, lat_hi);
   const BatchLattice &L = a.lats[lat];
@@ -320,13 +252,9 @@ __global__ void __launch_bounds__(MINB >= 5 ? 128 : kBatchMaxThreads, MINB)
   const uint32_t end = first + per < slots ? first + per : slots;
   const uint32_t slot = first + threadIdx.x;
   if (slot >= end) return;
-  const unsigned long long step = (unsigned long long)(*a.step_counter + k);
-  const float *rates = a.rates + 54 * lat;
-  char *pool = a.pool;
-  if (L.nx % 2 == 0)
-    batch_sites<D, PARITY, SHEAR, true, ROLLED>(L, pool, rates, slot, (uint32_t)step, (uint32_t)(step >> 32));
-  else
-    batch_sites<D, PARITY, SHEAR, false, ROLLED>(L, pool, rates, slot, (uint32_t)step, (uint32_t)(step >> 32));
+  const unsigned long long step = (unsigned long long)(*(volatile const long long *)a.step_counter + k);
+  batch_pair<D, PARITY, SHEAR, O, STAGE, THREADS>(L, PlaneStride{a.pool + 256ull * L.f256, 4ull * L.plane}, a.rates + 54 * lat,
+                                                  slot, step, early, stage + threadIdx.x);
 }
 
 // Advances the shared step counter after the n step launches of one call.
@@ -339,31 +267,54 @@ cudaError_t batch_max_blocks(bool shear, int threads, int *blocks_per_sm) {
                : cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, batch_kernel<false>, threads, 0);
 }
 
-// Launch shapes of the per-step form (BatchForm): register cap 128 (up to 256 threads,
-// two blocks per SM), or up to 128 threads with five (D3Q27, 102 registers) or ten (D2Q9,
-// 51 registers: its lighter update gains from the extra warps) blocks per SM; D3Q27
-// noise loop unrolled or rolled (D2Q9 has no loop).
-template <int D, bool SHEAR, int PARITY>
-cudaError_t launch_group(int form, const BatchArgs &a, int k, const BatchGroup &g, int threads, cudaStream_t s) {
+// Launch shapes of the per-step form (BatchForm): blocks of 128 threads per SM (as many threads in
+// other block sizes) that the kernel is compiled for, i.e. its register cap.
+template <int D>
+constexpr int batch_blocks(bool occ) {
+  return D == 2 ? (occ ? 10 : 8) : (occ ? 5 : 4);
+}
+
+template <int D, bool SHEAR, int PARITY, typename O>
+cudaError_t launch_group(int form, const BatchArgs &a, int k, const BatchGroup &g, int threads, bool dependent,
+                         cudaStream_t s) {
   if (g.ntiles <= 0) return cudaSuccess;
-  if (form == kBatchStepOcc)  // D3Q27: five blocks per SM; the lighter D2Q9 update: ten
-    batch_step_kernel<D, SHEAR, PARITY, false, D == 3 ? 5 : 10><<<g.ntiles, threads, 0, s>>>(a, k, g.lat_lo,
-                                                                                         g.lat_hi, g.tile0);
-  else if (form == kBatchStepRolled)  // D2Q9 has no noise loop: the same kernel as form 0
-    batch_step_kernel<D, SHEAR, PARITY, D == 3, 2><<<g.ntiles, threads, 0, s>>>(a, k, g.lat_lo, g.lat_hi, g.tile0);
-  else
-    batch_step_kernel<D, SHEAR, PARITY, false, 2><<<g.ntiles, threads, 0, s>>>(a, k, g.lat_lo, g.lat_hi, g.tile0);
-  return cudaGetLastError();
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(g.ntiles);
+  cfg.blockDim = dim3(threads);
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = dependent ? 1 : 0;
+  const bool early = (uint64_t)g.ntiles * (uint64_t)threads > kEarlySlots;
+  constexpr int B0 = batch_blocks<D>(false), B1 = batch_blocks<D>(true);
+  const auto launch = [&](auto kernel) {
+    return cudaLaunchKernelEx(&cfg, kernel, a, k, g.lat_lo, g.lat_hi, g.tile0, early);
+  };
+  if (threads == 256) return launch(batch_step_kernel<D, SHEAR, PARITY, O, 256, D == 2 ? 4 : 2>);
+  if (threads == 64)
+    return form == kBatchStepOcc ? launch(batch_step_kernel<D, SHEAR, PARITY, O, 64, 2 * B1>)
+                                 : launch(batch_step_kernel<D, SHEAR, PARITY, O, 64, 2 * B0>);
+  return form == kBatchStepOcc ? launch(batch_step_kernel<D, SHEAR, PARITY, O, 128, B1>)
+                               : launch(batch_step_kernel<D, SHEAR, PARITY, O, 128, B0>);
+}
+
+template <int D, bool SHEAR>
+cudaError_t launch_group_parity(int form, int parity, const BatchArgs &a, int k, const BatchGroup &g, int threads,
+                                bool dependent, cudaStream_t s) {
+  if (g.wide)
+    return parity ? launch_group<D, SHEAR, 1, uint64_t>(form, a, k, g, threads, dependent, s)
+                  : launch_group<D, SHEAR, 0, uint64_t>(form, a, k, g, threads, dependent, s);
+  return parity ? launch_group<D, SHEAR, 1, uint32_t>(form, a, k, g, threads, dependent, s)
+                : launch_group<D, SHEAR, 0, uint32_t>(form, a, k, g, threads, dependent, s);
 }
 
 template <int D>
 cudaError_t launch_group_any(int form, bool shear, int parity, const BatchArgs &a, int k, const BatchGroup &g,
-                             int threads, cudaStream_t s) {
-  if (shear)
-    return parity ? launch_group<D, true, 1>(form, a, k, g, threads, s)
-                  : launch_group<D, true, 0>(form, a, k, g, threads, s);
-  return parity ? launch_group<D, false, 1>(form, a, k, g, threads, s)
-                : launch_group<D, false, 0>(form, a, k, g, threads, s);
+                             int threads, bool dependent, cudaStream_t s) {
+  return shear ? launch_group_parity<D, true>(form, parity, a, k, g, threads, dependent, s)
+               : launch_group_parity<D, false>(form, parity, a, k, g, threads, dependent, s);
 }
 
 cudaError_t launch_batch_steps(int form3, int threads3, int form2, int threads2, bool shear, int parity0,
@@ -371,8 +322,9 @@ cudaError_t launch_batch_steps(int form3, int threads3, int form2, int threads2,
                                cudaStream_t s) {
   for (int k = 0; k < n; ++k) {
     const int parity = (parity0 + k) & 1;
-    cudaError_t e = launch_group_any<3>(form3, shear, parity, a, k, g3, threads3, s);
-    if (e == cudaSuccess) e = launch_group_any<2>(form2, shear, parity, a, k, g2, threads2, s);
+    cudaError_t e = launch_group_any<3>(form3, shear, parity, a, k, g3, threads3, k > 0, s);
+    if (e == cudaSuccess)
+      e = launch_group_any<2>(form2, shear, parity, a, k, g2, threads2, k > 0 || g3.ntiles > 0, s);
     if (e != cudaSuccess) return e;
   }
   batch_advance_kernel<<<1, 1, 0, s>>>(a.step_counter, n);

@@ -97,9 +97,10 @@ static_assert(sizeof(BatchArgs) <= 32764, "batch kernel arguments exceed the par
 cudaError_t batch_max_blocks(bool shear, int threads, int *blocks_per_sm);
 cudaError_t launch_batch(bool shear, const BatchArgs &a, int grid, int threads, cudaStream_t s);
 // The lattices of one type: table entries [lat_lo, lat_hi) owning tiles
-// [tile0, tile0 + ntiles).
+// [tile0, tile0 + ntiles); wide: a lattice of 4 GB or more among them (64-bit offsets).
 struct BatchGroup {
   int lat_lo, lat_hi, tile0, ntiles;
+  bool wide;
 };
 // Launch forms of a batch (values of flbm_batch_set_shape's `form`).
 enum BatchForm {

@@ -82,7 +82,28 @@ __host__ __device__ constexpr int stage_words() {
   return Lat<LAT>::Q + (sizeof(S) == 2 && PARITY == 1 ? (LAT == 2 ? 3 : 9) : 0);
 }
 
-template <int LAT, typename S, int PARITY, bool ALIGNED, bool ROWS, typename O, bool STAGE, int THREADS>
+// Address of byte `off` of population i's plane: from the planes' addresses in the kernel
+// arguments (the constant bank), or from a lattice's array and the bytes of its plane. In the
+// second form 32-bit offsets run over the whole array (below 4 GB), because i * plane in 64 bits
+// costs an access as much of the FMA pipe as four packed operations (batch of 32 D3Q27 64^3:
+// 0.307 ms a step with it, 0.281 with the 32-bit multiply-add, 0.313 with the planes' addresses
+// in shared memory).
+struct PlaneTable {
+  char *const *p;
+  template <typename O>
+  __device__ __forceinline__ char *at(int i, O off) const { return p[i] + (size_t)off; }
+};
+struct PlaneStride {
+  char *p;
+  unsigned long long plane;
+  __device__ __forceinline__ char *at(int i, uint32_t off) const {
+    return p + (size_t)(off + (uint32_t)i * (uint32_t)plane);
+  }
+  __device__ __forceinline__ char *at(int i, uint64_t off) const { return p + i * plane + off; }
+};
+
+template <int LAT, typename S, int PARITY, bool ALIGNED, bool ROWS, typename O, bool STAGE, int THREADS,
+          typename Base = PlaneTable>
 struct PairAccess {
   static constexpr int E = (int)sizeof(S);
   static constexpr int WORDS = stage_words<LAT, S, PARITY, ALIGNED, STAGE>();
@@ -90,7 +111,7 @@ struct PairAccess {
   using Word = typename std::conditional<E == 4, float2, uint32_t>::type;
   static_assert(!ROWS || (PARITY == 1 && ALIGNED), "rows of blocks are a form of the aligned odd step");
 
-  char *const *base;  // the populations' planes (kernel arguments: uniform addresses)
+  Base base;
   // Byte offsets in a plane. PARITY 0: x[1], x[2] the two lanes' sites. PARITY 1 aligned: x[1]
   // the pair at x0, x[2] the pair at x0 + 2; else x[0 .. 3] the sites x0 - 1 .. x0 + 2.
   O x[4];
@@ -99,8 +120,8 @@ struct PairAccess {
   uint32_t site0, dsite;   // local site index of lane x, and from it to lane y
 
   // PARITY 0: slot k of the range of n sites from `first`.
-  __device__ __forceinline__ void init_flat(char *const *pops, uint32_t first, uint32_t n, uint32_t k) {
-    base = pops;
+  __device__ __forceinline__ void init_flat(const Base &planes, uint32_t first, uint32_t n, uint32_t k) {
+    base = planes;
     site0 = first + 2u * k;
     two = ALIGNED || 2u * k + 1u < n;
     dsite = two ? 1u : 0u;
@@ -108,8 +129,8 @@ struct PairAccess {
     x[2] = x[1] + (two ? (O)E : (O)0);
   }
   // PARITY 1: the slot at (x0, y, z).
-  __device__ __forceinline__ void init_row(char *const *pops, int x0, int y, int z, int nx, int ny, int nz) {
-    base = pops;
+  __device__ __forceinline__ void init_row(const Base &planes, int x0, int y, int z, int nx, int ny, int nz) {
+    base = planes;
     const uint32_t row = ((uint32_t)z * (uint32_t)ny + (uint32_t)y) * (uint32_t)nx;
     if (ALIGNED) {
       const uint32_t s0 = row + (uint32_t)x0, s2 = row + (x0 + 2 == nx ? 0u : (uint32_t)x0 + 2u);
@@ -173,7 +194,7 @@ struct PairAccess {
     }
     return r;
   }
-  __device__ __forceinline__ char *at(int i, const Row &r, int k) const { return base[i] + (size_t)r.x[k]; }
+  __device__ __forceinline__ char *at(int i, const Row &r, int k) const { return base.at(i, r.x[k]); }
 
   // Starts the reads of the pair's arriving populations into the stage (at shared address
   // `st` of this thread's first word; words THREADS apart).

@@ -70,16 +70,16 @@ __global__ void __launch_bounds__(kStepBlock, MINB) pair_kernel(const StepArgs a
   if (ROWS) {
     const int x0 = 2 * (int)(blockIdx.x * kStepBlock + threadIdx.x);
     if (x0 >= a.nx) return;
-    p.init_row(a.pop, x0, blockIdx.y, blockIdx.z + a.z_lo, a.nx, a.ny, a.nz);
+    p.init_row(PlaneTable{a.pop}, x0, blockIdx.y, blockIdx.z + a.z_lo, a.nx, a.ny, a.nz);
   } else {
     const uint32_t slot = blockIdx.x * (uint32_t)kStepBlock + threadIdx.x;
     if (slot >= a.slots[PARITY]) return;
     if (PARITY == 0) {
-      p.init_flat(a.pop, a.first, a.count, slot);
+      p.init_flat(PlaneTable{a.pop}, a.first, a.count, slot);
     } else {
       int x0, y, z;
       slot_xyz(slot, a.nx, a.ny, a.m_hp, a.p_hp, a.m_ny, a.p_ny, x0, y, z);
-      p.init_row(a.pop, x0, y, z + a.z_lo, a.nx, a.ny, a.nz);
+      p.init_row(PlaneTable{a.pop}, x0, y, z + a.z_lo, a.nx, a.ny, a.nz);
     }
   }
   // Large launches: every read first, all of the noise while the populations travel. Small ones:

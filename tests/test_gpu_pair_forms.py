@@ -87,3 +87,48 @@ def test_forms_16_bit_one_step(fl, oracle_mod, storage, bits, lattice, dims):
             fo = oracle_mod.run(lattice, dims, lam, kbt, 5, f0, steps, 1)
             bound = np.abs(fo - w) * 2.0 ** -bits * 1.01 + 2e-6 * np.abs(fo) + 3e-8
             assert np.all(np.abs(fg - fo) <= bound), (rates, steps, kbt)
+
+
+def _streamed_match_oracle(lat, oracle_mod, lattice, dims, lam, kbt, seed, sites, advance, step):
+    """The oracle's collision of the sampled sites' populations against where one step put them."""
+    q = 9 if lattice == 0 else 27
+    c, w, _ = oracle_mod.tables(lattice)
+    pre = lat.sites_populations(sites)
+    advance()
+    worst = 0.0
+    for k, s in enumerate(sites):
+        x, y, z = s % dims[0], s // dims[0] % dims[1], s // (dims[0] * dims[1])
+        eta = oracle_mod.site_eta(lattice, seed, step, int(s))
+        fstar, _ = oracle_mod.collide_site(lattice, pre[k], lam, kbt, eta)
+        dest = ((x + c[:, 0]) % dims[0]) + dims[0] * (((y + c[:, 1]) % dims[1]) + dims[1] * ((z + c[:, 2]) % dims[2]))
+        got = lat.sites_populations(dest)[np.arange(q), np.arange(q)]
+        worst = max(worst, float((np.abs(got - fstar) / w).max()))
+    return worst
+
+
+def test_planes_of_4_gb(fl, oracle_mod):
+    # One plane of populations above 4 GB (64-bit offsets), both parities, corners included.
+    dims = (33000, 32770, 1)
+    n = dims[0] * dims[1]
+    sites = np.array([0, dims[0] - 1, n - 1, n - dims[0], n // 2 + 12345, (1 << 30) + 1, n - 70000])
+    with fl.Lattice(0, dims, _lam(9, "paper"), 1e-4, 1.0, 9) as lat:
+        lat.variant = 5
+        lat.init_uniform((0.03, 0.01, 0.0), 1e-3, 1)
+        for step in (0, 1):
+            assert _streamed_match_oracle(lat, oracle_mod, 0, dims, _lam(9, "paper"), 1e-4, 9, sites,
+                                          lambda: lat.step(1), step) <= TOL
+
+
+def test_batch_lattice_of_4_gb(fl, oracle_mod):
+    # A lattice whose array exceeds 4 GB (64-bit offsets in the batch kernel) beside a small one.
+    dims = (352, 340, 338)
+    n = dims[0] * dims[1] * dims[2]
+    specs = [dict(lattice=1, dims=dims, lam=_lam(27, "paper"), kBT=1e-4, rho0=1.0, seed=4),
+             dict(lattice=1, dims=(5, 4, 3), lam=_lam(27, "paper"), kBT=1e-4, rho0=1.0, seed=5)]
+    sites = np.array([0, dims[0] - 1, n - 1, n - dims[0], n // 2 + 12345, n - 70000])
+    with fl.Batch(specs) as b:
+        lat = b.lattice(0)
+        lat.init_uniform((0.03, 0.01, -0.02), 1e-3, 1)
+        for step in (0, 1):
+            assert _streamed_match_oracle(lat, oracle_mod, 1, dims, _lam(27, "paper"), 1e-4, 4, sites,
+                                          lambda: b.step(1), step) <= TOL
