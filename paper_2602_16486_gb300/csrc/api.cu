@@ -547,15 +547,17 @@ int flbm_fetch_samples(flbm_ctx *c, flbm_stats_t *out, int max_n, int *n_out) {
   DeviceGuard g(c->device);
   const int n = c->ring_count < max_n ? c->ring_count : max_n;
   const size_t len = size_t(stats_record_len(c->Q));
-  std::vector<double> h(len * size_t(n > 0 ? n : 1));
+  // One record (the members of an ensemble, sampled in turn) goes through the pinned mirror, more
+  // through pageable memory.
+  std::vector<double> many(n > 1 ? len * size_t(n) : 0);
+  double *h = n > 1 ? many.data() : c->h_acc;
   if (n > 0)
-    FLBM_CUDA(cudaMemcpyAsync(h.data(), c->d_ring, sizeof(double) * len * size_t(n),
-                              cudaMemcpyDeviceToHost, c->stream));
+    FLBM_CUDA(cudaMemcpyAsync(h, c->d_ring, sizeof(double) * len * size_t(n), cudaMemcpyDeviceToHost, c->stream));
   FLBM_CUDA(cudaStreamSynchronize(c->stream));
   int64_t bad = 0;
   bool timeout = false;
   for (int k = 0; k < n; ++k) {
-    fill_stats(c, h.data() + len * size_t(k), c->ring_steps[size_t(k)], &out[k]);
+    fill_stats(c, h + len * size_t(k), c->ring_steps[size_t(k)], &out[k]);
     if (out[k].nonfinite < 0)
       timeout = true;
     else

@@ -9,6 +9,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import threading
 
 import numpy as np
 
@@ -46,14 +47,22 @@ class flbm_stats_t(ctypes.Structure):
     ]
 
     def to_dict(self):
-        q = self.q
-        return {
-            "step": self.step, "sites": self.sites, "nonfinite": self.nonfinite,
-            "lattice": self.lattice, "q": q, "mass": self.mass,
-            "mom": np.array(self.mom[:]), "u_mean": np.array(self.u_mean[:]),
-            "uu": np.array(self.uu[:]), "k_mean": np.array(self.k_mean[:q]),
-            "k_cov": np.array(self.k_cov[:q * q]).reshape(q, q),
-        }
+        return _record_dict(np.frombuffer(self, dtype=np.float64))
+
+
+# The struct as doubles: three 64-bit and two 32-bit integers, then the floating-point fields.
+_RECORD_DOUBLES = ctypes.sizeof(flbm_stats_t) // 8
+
+
+def _record_dict(a):
+    """One record (a row of _RECORD_DOUBLES doubles) as a dict; the arrays are copies."""
+    step, sites, nonfinite = a[:3].view(np.int64).tolist()
+    lattice, q = a[3:4].view(np.int32).tolist()
+    return {
+        "step": step, "sites": sites, "nonfinite": nonfinite, "lattice": lattice, "q": q, "mass": float(a[4]),
+        "mom": a[5:8].copy(), "u_mean": a[8:11].copy(), "uu": a[11:17].copy(), "k_mean": a[17:17 + q].copy(),
+        "k_cov": a[44:44 + q * q].reshape(q, q).copy(),
+    }
 
 
 class flbm_lattice_spec(ctypes.Structure):
@@ -238,15 +247,30 @@ def flbm_sample(ctx):
     _check(_lib.flbm_sample(ctx))
 
 
+# Room for the records of one fetch, kept by each thread up to the default capacity (6.3 MB). Memory
+# of this size that is mapped and unmapped on every call costs 60-100 us, whatever is written to it.
+_KEPT_RECORDS = 1024
+_scratch = threading.local()
+
+
+def _record_buffer(n):
+    if n > _KEPT_RECORDS:
+        return np.empty((n, _RECORD_DOUBLES))
+    if not hasattr(_scratch, "records"):
+        _scratch.records = np.empty((_KEPT_RECORDS, _RECORD_DOUBLES))
+    return _scratch.records
+
+
 def flbm_fetch_samples(ctx, max_n=None, allow_nonfinite=False):
     cap = int(_lib.flbm_sample_capacity(ctx))
     max_n = cap if max_n is None else int(max_n)
-    buf = (flbm_stats_t * max(max_n, 1))()
+    buf = _record_buffer(max(max_n, 1))
     n = ctypes.c_int(0)
-    st = _lib.flbm_fetch_samples(ctx, buf, max_n, ctypes.byref(n))
+    st = _lib.flbm_fetch_samples(ctx, ctypes.cast(ctypes.c_void_p(buf.ctypes.data), ctypes.POINTER(flbm_stats_t)),
+                                 max_n, ctypes.byref(n))
     if not (st == FLBM_ENUMERIC and allow_nonfinite):
         _check(st)
-    return [buf[k].to_dict() for k in range(n.value)]
+    return [_record_dict(buf[k]) for k in range(n.value)]
 
 
 def flbm_set_sample_capacity(ctx, cap):
