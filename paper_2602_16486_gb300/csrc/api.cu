@@ -39,7 +39,9 @@ struct flbm_ctx {
   void *f = nullptr;
   bool own_f = false;
   size_t f_bytes = 0;
-  double *d_acc = nullptr;  // statistics accumulators (stats_record_len doubles)
+  // A statistics record (stats_record_len doubles), then the reduction's sums and ticket, zero between
+  // launches (stats.cu).
+  double *d_acc = nullptr;
   double *h_acc = nullptr;  // pinned host mirror of d_acc
   double *d_ring = nullptr;  // sample buffer: ring_cap records
   int ring_cap = 0, ring_count = 0;
@@ -295,11 +297,10 @@ int stats_result(const flbm_stats_t *out, long long step) {
   return FLBM_OK;
 }
 
-int enqueue_stats(flbm_ctx *c, double *acc_dev) {
-  FLBM_CUDA(cudaMemsetAsync(acc_dev, 0, sizeof(double) * stats_record_len(c->Q), c->stream));
-  FLBM_CUDA(launch_stats(klat(c->lattice), c->storage, c->iso, int(c->step & 1), c->f, c->N, int(c->dims[0]),
-                         int(c->dims[1]), int(c->dims[2]), float(c->rho0), acc_dev, c->stream, stat_site0(c),
-                         stat_sites(c)));
+int enqueue_stats(flbm_ctx *c, double *record) {
+  double *work = c->d_acc + stats_record_len(c->Q);
+  FLBM_CUDA(launch_stats(klat(c->lattice), c->storage, c->iso, int(c->step & 1), c->args, work,
+                         reinterpret_cast<unsigned int *>(work + stats_record_len(c->Q)), record, c->stream));
   return FLBM_OK;
 }
 
@@ -418,7 +419,9 @@ int flbm_create_ex(flbm_ctx **out, int lattice, const int64_t dims[3], const dou
     c->own_f = true;
   }
   const size_t acc_bytes = sizeof(double) * stats_record_len(c->Q);
-  e = cudaMalloc(&c->d_acc, acc_bytes);
+  const size_t work_bytes = 2 * acc_bytes + sizeof(double);
+  e = cudaMalloc(&c->d_acc, work_bytes);
+  if (e == cudaSuccess) e = cudaMemsetAsync(c->d_acc, 0, work_bytes, c->stream);
   if (e == cudaSuccess) e = cudaMallocHost(&c->h_acc, acc_bytes);
   if (e != cudaSuccess) {
     cudaGetLastError();
@@ -1463,19 +1466,21 @@ extern "C" int flbm_stats_noalloc(int lattice, const int64_t dims[3], int storag
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   const long long N = (long long)(dims[0] * dims[1] * dims[2]);
   FLBM_CUDA(cudaMemsetAsync(acc, 0, sizeof(double) * size_t(len), s));
-  FLBM_CUDA(launch_stats(klat(lattice), storage, lattice == FLBM_D3Q27_ISO, parity, dev_populations, N,
-                         int(dims[0]), int(dims[1]),
-                         int(dims[2]), float(rho0), acc, s, 0, N));
-  double h[FLBM_NOALLOC_SCRATCH_DOUBLES];
-  FLBM_CUDA(cudaMemcpyAsync(h, acc, sizeof(double) * size_t(len), cudaMemcpyDeviceToHost, s));
-  FLBM_CUDA(cudaStreamSynchronize(s));
-  // The host conversion of flbm_stats, fed with a description of this array.
+  // A description of this array, for the kernel's arguments and the host conversion of flbm_stats.
   flbm_ctx view;
   view.lattice = lattice;
   view.D = d_of(lattice);
   view.Q = Q;
   view.N = N;
+  for (int k = 0; k < 3; ++k) view.dims[k] = dims[k];
+  view.storage = storage;
   view.rho0 = rho0;
+  view.f = const_cast<void *>(dev_populations);
+  fill_args(&view);
+  FLBM_CUDA(launch_stats(klat(lattice), storage, lattice == FLBM_D3Q27_ISO, parity, view.args, nullptr, nullptr, acc, s));
+  double h[FLBM_NOALLOC_SCRATCH_DOUBLES];
+  FLBM_CUDA(cudaMemcpyAsync(h, acc, sizeof(double) * size_t(len), cudaMemcpyDeviceToHost, s));
+  FLBM_CUDA(cudaStreamSynchronize(s));
   fill_stats(&view, h, -1, out);
   return stats_result(out, -1);
 }

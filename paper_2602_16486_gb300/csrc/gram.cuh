@@ -278,14 +278,17 @@ struct Flush {
     taddr = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)((grow / P::ROWS) * P::ROWS);
     slot = grow / NC;
     i = grow % NC;
-    // Record entry e = a NC - a (a - 1) / 2 + (b - a) is G(a, b), a <= b (row-major upper
-    // triangle); this thread owns e = threadIdx.x + k kStatsBlock.
+    // Record entry e = S(a) + (b - a), S(a) = a NC - a (a - 1) / 2, is G(a, b), a <= b (row-major
+    // upper triangle); this thread owns e = threadIdx.x + k kStatsBlock. a by the quadratic, put
+    // right where the root is rounded.
 #pragma unroll
     for (int k = 0; k < PER_THREAD; ++k) {
       const int e = threadIdx.x + k * kStatsBlock;
-      int a = 0;
-      while (a + 1 < NC && (a + 1) * NC - (a + 1) * a / 2 <= e) ++a;
-      const int b = a + (e - (a * NC - a * (a - 1) / 2));
+      const auto start = [](int r) { return r * NC - r * (r - 1) / 2; };
+      int a = (int)(0.5f * ((float)(2 * NC + 1) - sqrtf((float)((2 * NC + 1) * (2 * NC + 1) - 8 * e))));
+      if (start(a) > e) --a;
+      if (start(a + 1) <= e) ++a;
+      const int b = a + (e - start(a));
       ent_off[k] = e < NREC ? b * NC + a : -1;
     }
   }

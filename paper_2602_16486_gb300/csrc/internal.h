@@ -147,10 +147,11 @@ cudaError_t launch_step_d3q19(int storage, int variant, int parity, bool noise, 
 // The raw-moment collision (step_raw.cu): D 2 or 3.
 cudaError_t launch_step_raw(int D, int storage, int variant, int parity, bool noise, const StepArgs &a,
                             cudaStream_t s);
-// Statistics of the sites [site0, site0 + nsites) of the array (the whole box: 0, plane).
-cudaError_t launch_stats(int D, int storage, bool iso, int parity, const void *f, long long plane, int nx,
-                         int ny, int nz, float rho0, double *acc, cudaStream_t s, long long site0,
-                         long long nsites);
+// Statistics of the sites a step of `a` would update (the whole box, or a slab's owned planes) to
+// the record `out`; work: stats_record_len zeros, zero again when the launch ends, and a ticket
+// counter likewise; or both null and `out` cleared beforehand.
+cudaError_t launch_stats(int D, int storage, bool iso, int parity, const StepArgs &a, double *work,
+                         unsigned int *ticket, double *out, cudaStream_t s);
 // site_base: global index of local site 0 (keys the density perturbation).
 cudaError_t launch_init(int D, int storage, void *f, long long plane, int nx, int ny, int nz,
                         double rho0, double ux, double uy, double uz, double amp,

@@ -7,9 +7,17 @@
 // (gram.cuh: staging layout, BF16 hi/lo products on the tcgen05 tensor cores with a TMEM
 // accumulator, output record; k_0 = rho and the central moments k_1..k_D, which vanish
 // identically, are rebuilt or set to zero by the host, api.cu). Persistent blocks of
-// kStatsBlock threads walk tiles of 2 kStatsBlock sites: each thread computes the columns
-// of two sites with the packed FP32x2 algebra of the step (cm.cuh) and writes their BF16
-// hi/lo words into its warp's operand rows; one thread per block multiplies the tile.
+// kStatsBlock threads walk tiles of kStatsBlock site pairs, the flat pairs of the step kernels
+// (pair.cuh): each thread computes the columns of two sites with the packed FP32x2 algebra of
+// the step (cm.cuh) and writes their BF16 hi/lo words into its warp's operand rows; one thread
+// per block multiplies the tile.
+// What bounds it: three warps per scheduler (168 registers with the next pair's populations in
+// flight) on long chains of packed operations and conversions, 50 % of issue slots, DRAM half busy;
+// on small lattices the chain of set-up, one tile, accumulator read and block sums.
+// us per sample, before -> now: D3Q27 256^3 421 -> 369 (even step count), 433 -> 406 (odd), 255^3 568 ->
+// 422 / 454, 64^3 21.9 -> 20.0; D3Q19 256^3 410 -> 360; D2Q9 4096^2 165 -> 143, 64^2 9.0 -> 6.6. The
+// planes' addresses as kernel arguments and one division per pair gave the large ones, no clearing
+// launch and the set-up before the wait the small ones.
 #include <cuda_runtime.h>
 
 #include <map>
@@ -20,6 +28,7 @@
 #include "d3q19.cuh"
 #include "gram.cuh"
 #include "internal.h"
+#include "pair.cuh"
 
 namespace flbm {
 
@@ -27,60 +36,48 @@ int stats_nacc(int Q) { return Q == 9 ? StatsPlan<2>::NREC : StatsPlan<3>::NREC;
 
 namespace {
 
-using gram::kTileSites;
-
 // The populations of a thread's site pair, as loaded for one tile and consumed by the
 // next: F19 for D3Q19 (lattice code 19), the 3x3x3 tile otherwise.
 template <int D>
 struct PairPops {
   float2 F[3][3][3];
+  bool v0, v1;  // the lanes' sites exist
 };
 template <>
 struct PairPops<19> {
   float2 F[19];
+  bool v0, v1;
 };
 
-// Loads the pair's populations (lane x: site s, lane y: site s + 1; zeros for a site
-// beyond N). PAIRROW: nx is even, so s (even) and s + 1 share a row and load as pairs; on
-// odd parity the pair is the step's (cm.cuh, load_pairs: sites s + 1 and s + 2 of the
-// row), which covers the same sites.
-template <int D, typename S, int PARITY, bool PAIRROW>
-__device__ __forceinline__ void load_pair(const S *__restrict__ f, long long plane, int nx, int ny, int nz,
-                                          long long s, long long N, PairPops<D> &P) {
-  constexpr int NP = D == 19 ? 19 : 27;
+// Loads the pair of slot k (the slots of the step kernels, pair.cuh, of the sites the statistics
+// cover); zeros for a lane without a site of its own.
+template <int LAT, typename S, int PARITY, bool ALIGNED>
+__device__ __forceinline__ void load_pair(const StepArgs &a, uint32_t k, PairPops<LAT> &P) {
+  constexpr int NP = LAT == 2 ? 27 : Lat<LAT>::Q;  // D2Q9 uses the middle plane of its tile
   float2 *F = reinterpret_cast<float2 *>(&P.F);
-  if (PAIRROW) {
-    if (s < N) {
-      const uint32_t r = (uint32_t)s / (uint32_t)nx, q = r / (uint32_t)ny;
-      const int x0 = (int)((uint32_t)s - r * (uint32_t)nx), y = (int)(r - q * (uint32_t)ny), z = (int)q;
-      if constexpr (D == 19)
-        load19_pairs<S, PARITY>(f, plane, addr2(x0, y, z, nx, ny, nz), P.F);
-      else
-        load_pairs<D, S, PARITY>(f, plane, addr2(x0, y, z, nx, ny, nz), P.F);
+  P.v0 = k < a.slots[PARITY];
+  P.v1 = false;
+  if (P.v0) {
+    PairAccess<LAT, S, PARITY, ALIGNED, false, uint64_t, false, 1> p;
+    if (PARITY == 0) {
+      p.init_flat(PlaneTable{a.pop}, a.first, a.count, k);
     } else {
+      int x0, y, z;
+      slot_xyz(k, a.nx, a.ny, a.m_hp, a.p_hp, a.m_ny, a.p_ny, x0, y, z);
+      p.init_row(PlaneTable{a.pop}, x0, y, z + a.z_lo, a.nx, a.ny, a.nz);
+    }
+    if constexpr (LAT == 19)
+      p.load_list(nullptr, P.F);
+    else
+      p.load_tile(nullptr, P.F);
+    P.v1 = p.two;
+    if (!ALIGNED && !p.two) {
 #pragma unroll
-      for (int a = 0; a < NP; ++a) F[a] = make_float2(0.0f, 0.0f);
+      for (int q = 0; q < NP; ++q) F[q].y = 0.0f;
     }
   } else {
 #pragma unroll
-    for (int l = 0; l < 2; ++l) {
-      const long long sl = s + l;
-      float Fl[NP];
-      if (sl < N) {
-        const uint32_t r = (uint32_t)sl / (uint32_t)nx, q = r / (uint32_t)ny;
-        const int x = (int)((uint32_t)sl - r * (uint32_t)nx), y = (int)(r - q * (uint32_t)ny), z = (int)q;
-        if constexpr (D == 19)
-          load19<S, PARITY>(f, plane, neighbourhood(x, y, z, nx, ny, nz), Fl);
-        else
-          load_logical<D, S, PARITY>(f, plane, neighbourhood(x, y, z, nx, ny, nz),
-                                     *reinterpret_cast<float(*)[3][3][3]>(Fl));
-      } else {
-#pragma unroll
-        for (int a = 0; a < NP; ++a) Fl[a] = 0.0f;
-      }
-#pragma unroll
-      for (int a = 0; a < NP; ++a) set_lane(F[a], l, Fl[a]);
-    }
+    for (int q = 0; q < NP; ++q) F[q] = make_float2(0.0f, 0.0f);
   }
 }
 
@@ -125,41 +122,56 @@ __device__ __forceinline__ void pair_columns(PairPops<D> &P, float rho0, bool v0
   }
 }
 
-// One block walks tiles of kTileSites sites: every thread transforms its site pair
+// One block walks tiles of kStatsBlock pairs: every thread transforms its site pair
 // (loaded during the previous tile) and stages the split columns; each warp then arrives
 // once on the pipeline's "staged" mbarrier and thread 0 multiplies the tile (gram.cuh,
 // Pipeline). Before a thread overwrites the staging rows it waits for the MMAs that read
 // them (one phase of each mbarrier per tile; every wait bounded), so the loads and
 // arithmetic of the next tile proceed while the tensor cores work.
-template <int D, typename S, int PARITY, bool PAIRROW, bool ISO>
-__global__ void __launch_bounds__(kStatsBlock, gram::blocks_per_sm<D>()) stats_kernel(const S *__restrict__ f, long long plane,
-                                                               int nx, int ny, int nz, float rho0,
-                                                               double *__restrict__ out, long long site0,
-                                                               long long site1) {
-  constexpr int NC = StatsPlan<D>::NC;
+// The set-up (TMEM, barriers, tables) runs before the wait for the launch before this one
+// (programmatic dependent launch). The blocks' sums meet in `work`, which is zero between
+// launches: the last block to finish moves them to the record `out` and clears them, so that a
+// sample is one launch with no clearing before it. Without `work` they are added to `out`, cleared
+// by the caller.
+template <int LAT, typename S, int PARITY, bool ALIGNED, bool ISO>
+__global__ void __launch_bounds__(kStatsBlock, gram::blocks_per_sm<LAT>())
+    stats_kernel(const StepArgs a, uint32_t tiles, double *work, unsigned int *ticket, double *out) {
+  constexpr int NC = StatsPlan<LAT>::NC;
   extern __shared__ unsigned char smem_raw[];
   __shared__ unsigned int flags[2];  // non-finite count of the block, failure flag
-  gram::Pipeline<D> pl;
+  gram::Pipeline<LAT> pl;
   pl.init(smem_raw, flags);
+  wait_prerequisites();
 
   unsigned nonfinite = 0u;
-  const long long N = site1;  // sites [site0, site1) of the array (plane = its Q-stride)
-  const long long stride = (long long)gridDim.x * kTileSites;
   // Software pipelining: the populations of the thread's pair in the next tile are loaded
   // as soon as the current ones are consumed, so the loads are in flight while the thread
   // splits and stages its columns and waits for the tensor cores.
-  PairPops<D> pp;
-  if (site0 + (long long)blockIdx.x * kTileSites < N)
-    load_pair<D, S, PARITY, PAIRROW>(f, plane, nx, ny, nz, site0 + (long long)blockIdx.x * kTileSites + 2 * threadIdx.x,
-                                     N, pp);
-  for (long long base = site0 + (long long)blockIdx.x * kTileSites; base < N; base += stride) {
-    const long long s = base + 2 * threadIdx.x;
+  PairPops<LAT> pp;
+  load_pair<LAT, S, PARITY, ALIGNED>(a, blockIdx.x * (uint32_t)kStatsBlock + threadIdx.x, pp);
+  for (uint32_t t = blockIdx.x; t < tiles; t += gridDim.x) {
     float2 col[NC];
-    pair_columns<D, ISO>(pp, rho0, s < N, s + 1 < N, col, nonfinite);
-    if (base + stride < N) load_pair<D, S, PARITY, PAIRROW>(f, plane, nx, ny, nz, s + stride, N, pp);
+    pair_columns<LAT, ISO>(pp, a.rho0, pp.v0, pp.v1, col, nonfinite);
+    if (t + gridDim.x < tiles)
+      load_pair<LAT, S, PARITY, ALIGNED>(a, (t + gridDim.x) * (uint32_t)kStatsBlock + threadIdx.x, pp);
     pl.tile(col);
   }
-  pl.end(nonfinite, flags, out);
+  // Only now: blocks of the next step that wait beside a long reduction take its L1 cache
+  // (256^3 sample between steps 0.52 against 0.39 ms).
+  launch_dependents();
+  pl.end(nonfinite, flags, work ? work : out);
+  if (work == nullptr) return;
+  __threadfence();  // this block's sums before its ticket
+  __syncthreads();
+  if (threadIdx.x == 0) flags[0] = atomicAdd(ticket, 1u) == gridDim.x - 1 ? 1u : 0u;
+  __syncthreads();
+  if (flags[0] == 0u) return;
+  __threadfence();
+  for (int e = threadIdx.x; e <= StatsPlan<LAT>::NREC; e += kStatsBlock) {
+    out[e] = __ldcg(work + e);
+    work[e] = 0.0;
+  }
+  if (threadIdx.x == 0) *ticket = 0u;
 }
 
 template <int D, typename S>
@@ -193,60 +205,57 @@ cudaError_t stats_grid(K kernel, size_t smem, long long tiles, int per_sm, int *
   return cudaSuccess;
 }
 
-template <int D, typename S, int PARITY, bool PAIRROW, bool ISO>
-cudaError_t launch_one(const S *p, long long plane, int nx, int ny, int nz, float rho0, double *acc,
-                       cudaStream_t s, long long site0, long long nsites) {
-  auto kernel = stats_kernel<D, S, PARITY, PAIRROW, ISO>;
-  const size_t smem = stats_smem<D, S>();
-  const long long tiles = (nsites + kTileSites - 1) / kTileSites;
+template <int LAT, typename S, int PARITY, bool ALIGNED, bool ISO>
+cudaError_t launch_one(const StepArgs &a, double *work, unsigned int *ticket, double *out, cudaStream_t s) {
+  auto kernel = stats_kernel<LAT, S, PARITY, ALIGNED, ISO>;
+  const size_t smem = stats_smem<LAT, S>();
+  const uint32_t tiles = (uint32_t)(((uint64_t)a.slots[PARITY] + kStatsBlock - 1) / kStatsBlock);
   if (tiles == 0) return cudaSuccess;
   int grid = 0;
-  const cudaError_t e = stats_grid(kernel, smem, tiles, gram::blocks_per_sm<D>(), &grid);
+  const cudaError_t e = stats_grid(kernel, smem, tiles, gram::blocks_per_sm<LAT>(), &grid);
   if (e != cudaSuccess) return e;
-  kernel<<<grid, kStatsBlock, smem, s>>>(p, plane, nx, ny, nz, rho0, acc, site0, site0 + nsites);
-  return cudaGetLastError();
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(kStatsBlock);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  // Blocks that arrive beside a draining step find the SM's memory split as that kernel left it and
+  // may not all fit; where each block has many tiles that costs more than the early start gives
+  // (D3Q27 256^3, 144 tiles a block, sample between steps 0.48 against 0.39 ms; 128^3, 18 tiles,
+  // 61.8 against 61.4 us; 64^3, 2 tiles, 20.1 against 21.4).
+  cfg.numAttrs = tiles > 8u * (uint32_t)grid ? 0 : 1;
+  return cudaLaunchKernelEx(&cfg, kernel, a, tiles, work, ticket, out);
 }
 
-template <int D, typename S, bool ISO>
-cudaError_t launch_typed(int parity, const void *f, long long plane, int nx, int ny, int nz,
-                         float rho0, double *acc, cudaStream_t s, long long site0, long long nsites) {
-  const S *p = static_cast<const S *>(f);
-  // Pairs (s, s + 1) share a row when nx is even and every tile starts on an even site.
-  const bool pairrow = nx % 2 == 0 && site0 % 2 == 0;
+template <int LAT, typename S, bool ISO>
+cudaError_t launch_typed(int parity, const StepArgs &a, double *work, unsigned int *ticket, double *out, cudaStream_t s) {
   if (parity == 0)
-    return pairrow ? launch_one<D, S, 0, true, ISO>(p, plane, nx, ny, nz, rho0, acc, s, site0, nsites)
-                   : launch_one<D, S, 0, false, ISO>(p, plane, nx, ny, nz, rho0, acc, s, site0, nsites);
-  return pairrow ? launch_one<D, S, 1, true, ISO>(p, plane, nx, ny, nz, rho0, acc, s, site0, nsites)
-                 : launch_one<D, S, 1, false, ISO>(p, plane, nx, ny, nz, rho0, acc, s, site0, nsites);
+    return a.aligned[0] ? launch_one<LAT, S, 0, true, ISO>(a, work, ticket, out, s)
+                        : launch_one<LAT, S, 0, false, ISO>(a, work, ticket, out, s);
+  return a.aligned[1] ? launch_one<LAT, S, 1, true, ISO>(a, work, ticket, out, s)
+                      : launch_one<LAT, S, 1, false, ISO>(a, work, ticket, out, s);
+}
+
+template <int LAT, bool ISO>
+cudaError_t launch_storage(int storage, int parity, const StepArgs &a, double *work, unsigned int *ticket, double *out,
+                           cudaStream_t s) {
+  if (storage == 0) return launch_typed<LAT, float, ISO>(parity, a, work, ticket, out, s);
+  if (storage == 1) return launch_typed<LAT, __nv_bfloat16, ISO>(parity, a, work, ticket, out, s);
+  return launch_typed<LAT, __half, ISO>(parity, a, work, ticket, out, s);
 }
 
 }  // namespace
 
-cudaError_t launch_stats(int D, int storage, bool iso, int parity, const void *f, long long plane, int nx,
-                         int ny, int nz, float rho0, double *acc, cudaStream_t s, long long site0,
-                         long long nsites) {
-  if (D == 19) {  // D3Q19 (lattice code 19)
-    if (storage == 0) return launch_typed<19, float, false>(parity, f, plane, nx, ny, nz, rho0, acc, s, site0, nsites);
-    if (storage == 1)
-      return launch_typed<19, __nv_bfloat16, false>(parity, f, plane, nx, ny, nz, rho0, acc, s, site0, nsites);
-    return launch_typed<19, __half, false>(parity, f, plane, nx, ny, nz, rho0, acc, s, site0, nsites);
-  }
-  if (D == 3 && iso) {
-    if (storage == 0) return launch_typed<3, float, true>(parity, f, plane, nx, ny, nz, rho0, acc, s, site0, nsites);
-    if (storage == 1)
-      return launch_typed<3, __nv_bfloat16, true>(parity, f, plane, nx, ny, nz, rho0, acc, s, site0, nsites);
-    return launch_typed<3, __half, true>(parity, f, plane, nx, ny, nz, rho0, acc, s, site0, nsites);
-  }
-  if (D == 3) {
-    if (storage == 0) return launch_typed<3, float, false>(parity, f, plane, nx, ny, nz, rho0, acc, s, site0, nsites);
-    if (storage == 1)
-      return launch_typed<3, __nv_bfloat16, false>(parity, f, plane, nx, ny, nz, rho0, acc, s, site0, nsites);
-    return launch_typed<3, __half, false>(parity, f, plane, nx, ny, nz, rho0, acc, s, site0, nsites);
-  }
-  if (storage == 0) return launch_typed<2, float, false>(parity, f, plane, nx, ny, nz, rho0, acc, s, site0, nsites);
-  if (storage == 1)
-    return launch_typed<2, __nv_bfloat16, false>(parity, f, plane, nx, ny, nz, rho0, acc, s, site0, nsites);
-  return launch_typed<2, __half, false>(parity, f, plane, nx, ny, nz, rho0, acc, s, site0, nsites);
+cudaError_t launch_stats(int D, int storage, bool iso, int parity, const StepArgs &a, double *work,
+                         unsigned int *ticket, double *out, cudaStream_t s) {
+  if (D == 19) return launch_storage<19, false>(storage, parity, a, work, ticket, out, s);
+  if (D == 2) return launch_storage<2, false>(storage, parity, a, work, ticket, out, s);
+  return iso ? launch_storage<3, true>(storage, parity, a, work, ticket, out, s)
+             : launch_storage<3, false>(storage, parity, a, work, ticket, out, s);
 }
 
 }  // namespace flbm
