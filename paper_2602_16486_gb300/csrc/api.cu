@@ -238,7 +238,6 @@ int ensure_stage(flbm_ctx *c, size_t elems) {
 // then the non-finite count. k_0 = rho = rho0 + (rho - rho0) is rebuilt in FP64; the
 // central moments k_1..k_D vanish identically and are reported as 0.
 // Sites the statistics cover: the whole box, or a slab's owned planes.
-long long stat_site0(const flbm_ctx *c) { return c->slab ? (long long)(c->dims[0] * c->dims[1]) : 0; }
 long long stat_sites(const flbm_ctx *c) {
   return c->slab ? (long long)(c->dims[0] * c->dims[1] * c->z_count) : c->N;
 }

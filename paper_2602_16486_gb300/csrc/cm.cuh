@@ -58,30 +58,12 @@ __device__ __forceinline__ void raw_fwd(T &p0, T &p1, T &p2) {
   p0 = s;
 }
 
-// Inverse of raw_fwd.
-template <typename T>
-__device__ __forceinline__ void raw_inv(T &p0, T &p1, T &p2) {
-  const T s = p0, d = p1;
-  const T e = vfma(splat<T>(kCs2), s, p2);
-  p1 = vsub(s, e);
-  p2 = vmul(splat<T>(0.5f), vadd(e, d));
-  p0 = vmul(splat<T>(0.5f), vsub(e, d));
-}
-
 // Raw -> central moments along one axis; nu = -u (velocity component, negated).
 template <typename T>
 __device__ __forceinline__ void shift_fwd(T &m0, T &m1, T &m2, T nu) {
   const T k1 = vfma(nu, m0, m1);
   m2 = vfma(nu, vadd(m1, k1), m2);
   m1 = k1;
-}
-
-// Central -> raw moments along one axis (inverse of shift_fwd), velocity component u.
-template <typename T>
-__device__ __forceinline__ void shift_inv(T &k0, T &k1, T &k2, T u) {
-  const T r1 = vfma(u, k0, k1);
-  k2 = vfma(u, vadd(k1, r1), k2);
-  k1 = r1;
 }
 
 // The inverses in the halved convention: along the transformed axis the slots of order 1
@@ -125,25 +107,6 @@ __device__ __forceinline__ void tile_raw_fwd(T (&F)[3][3][3]) {
   }
 }
 
-template <int D, typename T>
-__device__ __forceinline__ void tile_raw_inv(T (&F)[3][3][3]) {
-  constexpr int z0 = (D == 3) ? 0 : 1, z1 = (D == 3) ? 3 : 2;
-  if (D == 3) {
-#pragma unroll
-    for (int b = 0; b < 3; ++b)
-#pragma unroll
-      for (int a = 0; a < 3; ++a) raw_inv(F[0][b][a], F[1][b][a], F[2][b][a]);
-  }
-#pragma unroll
-  for (int z = z0; z < z1; ++z)
-#pragma unroll
-    for (int a = 0; a < 3; ++a) raw_inv(F[z][0][a], F[z][1][a], F[z][2][a]);
-#pragma unroll
-  for (int z = z0; z < z1; ++z)
-#pragma unroll
-    for (int y = 0; y < 3; ++y) raw_inv(F[z][y][0], F[z][y][1], F[z][y][2]);
-}
-
 // Central shift of all moments with the negated velocity (nux, nuy, nuz).
 template <int D, typename T>
 __device__ __forceinline__ void tile_shift_fwd(T (&F)[3][3][3], T nux, T nuy, T nuz) {
@@ -162,25 +125,6 @@ __device__ __forceinline__ void tile_shift_fwd(T (&F)[3][3][3], T nux, T nuy, T 
 #pragma unroll
       for (int a = 0; a < 3; ++a) shift_fwd(F[0][b][a], F[1][b][a], F[2][b][a], nuz);
   }
-}
-
-template <int D, typename T>
-__device__ __forceinline__ void tile_shift_inv(T (&F)[3][3][3], T ux, T uy, T uz) {
-  constexpr int z0 = (D == 3) ? 0 : 1, z1 = (D == 3) ? 3 : 2;
-  if (D == 3) {
-#pragma unroll
-    for (int b = 0; b < 3; ++b)
-#pragma unroll
-      for (int a = 0; a < 3; ++a) shift_inv(F[0][b][a], F[1][b][a], F[2][b][a], uz);
-  }
-#pragma unroll
-  for (int z = z0; z < z1; ++z)
-#pragma unroll
-    for (int a = 0; a < 3; ++a) shift_inv(F[z][0][a], F[z][1][a], F[z][2][a], uy);
-#pragma unroll
-  for (int z = z0; z < z1; ++z)
-#pragma unroll
-    for (int b = 0; b < 3; ++b) shift_inv(F[z][b][0], F[z][b][1], F[z][b][2], ux);
 }
 
 // Inverses of the whole tile in the halved convention (tile_scale in lattice.cuh): central
@@ -230,27 +174,6 @@ __device__ __forceinline__ void tile_raw_inv_h(T (&F)[3][3][3]) {
 template <int D, typename T>
 __device__ __forceinline__ T &mom(T (&F)[3][3][3], int a, int b, int c) {
   return D == 3 ? F[c][b][a] : F[1][b][a];
-}
-
-// Central moments of one site in the paper's mode order (Sec. II-B / II-C), from the
-// tile after tile_shift_fwd with entry (0,0,0) = rho.
-template <int D>
-__device__ __forceinline__ void paper_modes(float (&F)[3][3][3], float *k) {
-  if (D == 3) {
-#pragma unroll
-    for (int v = 0; v < 27; ++v) {
-      const int t = d3q27_mode_tensor(v);
-      k[v] = F[t / 9][(t / 3) % 3][t % 3];
-    }
-  } else {
-#pragma unroll
-    for (int v = 0; v < 9; ++v) {
-      const int t = d2q9_mode_tensor(v);
-      if (t >= 0) k[v] = F[1][t / 3][t % 3];
-    }
-    k[3] = F[1][0][2] + F[1][2][0];
-    k[4] = F[1][0][2] - F[1][2][0];
-  }
 }
 
 // ---- periodic neighbourhood and AA-pattern addressing -----------------------------------
@@ -319,9 +242,7 @@ __device__ __forceinline__ void store_streamed(S *__restrict__ f, long long plan
       }
 }
 
-// ---- two sites per thread: x0 and x0 + 1 (x0 even, nx even) ------------------------------
-// Pair loads/stores of two consecutive x; the array is 2-element aligned because nx is
-// even and the buffer is 256-byte aligned.
+// ---- two sites per thread (pair.cuh): loads and stores of two consecutive, aligned elements -------
 template <typename S>
 struct Storage2;
 template <>
@@ -349,163 +270,6 @@ struct Storage2<__half> {
     *reinterpret_cast<__half2 *>(p) = __floats2half2_rn(v.x, v.y);
   }
 };
-
-// Site indices of a thread's pair and the periodic row / plane offsets of its block.
-// y and z are fixed per block, so dy and dz are the same for every thread of it; only
-// s0, sm1 and sp2 (the x seam) vary between threads.
-struct Addr2 {
-  long long s0;          // site x0
-  long long sm1, sp2;    // sites x0 - 1 and x0 + 2 of the same row (periodic)
-  long long dy[3];       // offset of row y - 1, y, y + 1 (periodic)
-  long long dz[3];       // offset of plane z - 1, z, z + 1 (periodic)
-};
-
-__device__ __forceinline__ Addr2 addr2(int x0, int y, int z, int nx, int ny, int nz) {
-  Addr2 a;
-  a.s0 = ((long long)z * ny + y) * nx + x0;
-  a.sm1 = a.s0 + (x0 == 0 ? nx - 1 : -1);
-  a.sp2 = a.s0 + (x0 + 2 == nx ? 2 - nx : 2);
-  const long long row = nx, pl = (long long)nx * ny;
-  a.dy[0] = (y == 0) ? (long long)(ny - 1) * row : -row;
-  a.dy[1] = 0;
-  a.dy[2] = (y == ny - 1) ? -(long long)(ny - 1) * row : row;
-  a.dz[0] = (z == 0) ? (long long)(nz - 1) * pl : -pl;
-  a.dz[1] = 0;
-  a.dz[2] = (z == nz - 1) ? -(long long)(nz - 1) * pl : pl;
-  return a;
-}
-
-// As load_logical, for the pair: lane x holds site x0, lane y site x0 + 1.
-template <int D, typename S, int PARITY>
-__device__ __forceinline__ void load_logical2(const S *__restrict__ f, long long plane, const Addr2 &ad,
-                                              float2 (&F)[3][3][3]) {
-  constexpr int z0 = (D == 3) ? -1 : 0, z1 = (D == 3) ? 1 : 0;
-#pragma unroll
-  for (int dz = z0; dz <= z1; ++dz)
-#pragma unroll
-    for (int dy = -1; dy <= 1; ++dy)
-#pragma unroll
-      for (int dx = -1; dx <= 1; ++dx) {
-        const int i = Lat<D>::index(dx, dy, dz);
-        float2 v;
-        if (PARITY == 0) {
-          v = Storage2<S>::load(f + i * plane + ad.s0);
-        } else {
-          // f_i(x) = A[opposite(i)][x - c_i]
-          const S *b = f + opposite<D>(i) * plane + ad.dy[1 - dy] + ad.dz[1 - dz];
-          if (dx == 0) {
-            v = Storage2<S>::load(b + ad.s0);
-          } else if (dx == 1) {
-            v.x = Storage<S>::load(b + ad.sm1);
-            v.y = Storage<S>::load(b + ad.s0);
-          } else {
-            v.x = Storage<S>::load(b + ad.s0 + 1);
-            v.y = Storage<S>::load(b + ad.sp2);
-          }
-        }
-        F[dz + 1][dy + 1][dx + 1] = v;
-      }
-}
-
-// As store_streamed, for the pair.
-template <int D, typename S, int PARITY>
-__device__ __forceinline__ void store_streamed2(S *__restrict__ f, long long plane, const Addr2 &ad,
-                                                const float2 (&F)[3][3][3]) {
-  constexpr int z0 = (D == 3) ? -1 : 0, z1 = (D == 3) ? 1 : 0;
-#pragma unroll
-  for (int dz = z0; dz <= z1; ++dz)
-#pragma unroll
-    for (int dy = -1; dy <= 1; ++dy)
-#pragma unroll
-      for (int dx = -1; dx <= 1; ++dx) {
-        const int i = Lat<D>::index(dx, dy, dz);
-        const float2 v = F[dz + 1][dy + 1][dx + 1];
-        if (PARITY == 0) {
-          Storage2<S>::store(f + opposite<D>(i) * plane + ad.s0, v);
-        } else {
-          // f*_i(x) goes to A[i][x + c_i]
-          S *b = f + i * plane + ad.dy[1 + dy] + ad.dz[1 + dz];
-          if (dx == 0) {
-            Storage2<S>::store(b + ad.s0, v);
-          } else if (dx == 1) {
-            Storage<S>::store(b + ad.s0 + 1, v.x);
-            Storage<S>::store(b + ad.sp2, v.y);
-          } else {
-            Storage<S>::store(b + ad.sm1, v.x);
-            Storage<S>::store(b + ad.s0, v.y);
-          }
-        }
-      }
-}
-
-// Pairs of the step kernels: on even steps (PARITY 0) lane x holds site x0 and lane y site
-// x0 + 1; on odd steps lane x holds x0 + 1 and lane y x0 + 2, which is the row's first site
-// when x0 + 2 = nx (ad.sp2). An odd step reads slot opposite(i) at x - c_i and writes slot i
-// at x + c_i, so with this pairing the populations with c_x = +-1 (18 of 27 on D3Q27) move as
-// aligned pairs, (x0, x0 + 1) or (x0 + 2, x0 + 3), and only those with c_x = 0 take two scalar
-// accesses. Every site of a row is still covered once.
-template <int D, typename S, int PARITY>
-__device__ __forceinline__ void load_pairs(const S *__restrict__ f, long long plane, const Addr2 &ad,
-                                           float2 (&F)[3][3][3]) {
-  if (PARITY == 0) {
-    load_logical2<D, S, 0>(f, plane, ad, F);
-    return;
-  }
-  constexpr int z0 = (D == 3) ? -1 : 0, z1 = (D == 3) ? 1 : 0;
-#pragma unroll
-  for (int dz = z0; dz <= z1; ++dz)
-#pragma unroll
-    for (int dy = -1; dy <= 1; ++dy)
-#pragma unroll
-      for (int dx = -1; dx <= 1; ++dx) {
-        const int i = Lat<D>::index(dx, dy, dz);
-        const S *b = f + opposite<D>(i) * plane + ad.dy[1 - dy] + ad.dz[1 - dz];  // row of x - c_i
-        float2 v;
-        if (dx == 0) {
-          v.x = Storage<S>::load(b + ad.s0 + 1);
-          v.y = Storage<S>::load(b + ad.sp2);
-        } else {
-          v = Storage2<S>::load(b + (dx == 1 ? ad.s0 : ad.sp2));
-        }
-        F[dz + 1][dy + 1][dx + 1] = v;
-      }
-}
-
-template <int D, typename S, int PARITY>
-__device__ __forceinline__ void store_pairs(S *__restrict__ f, long long plane, const Addr2 &ad,
-                                            const float2 (&F)[3][3][3]) {
-  if (PARITY == 0) {
-    store_streamed2<D, S, 0>(f, plane, ad, F);
-    return;
-  }
-  constexpr int z0 = (D == 3) ? -1 : 0, z1 = (D == 3) ? 1 : 0;
-#pragma unroll
-  for (int dz = z0; dz <= z1; ++dz)
-#pragma unroll
-    for (int dy = -1; dy <= 1; ++dy)
-#pragma unroll
-      for (int dx = -1; dx <= 1; ++dx) {
-        const int i = Lat<D>::index(dx, dy, dz);
-        S *b = f + i * plane + ad.dy[1 + dy] + ad.dz[1 + dz];  // row of x + c_i
-        const float2 v = F[dz + 1][dy + 1][dx + 1];
-        if (dx == 0) {
-          Storage<S>::store(b + ad.s0 + 1, v.x);
-          Storage<S>::store(b + ad.sp2, v.y);
-        } else {
-          Storage2<S>::store(b + (dx == 1 ? ad.sp2 : ad.s0), v);
-        }
-      }
-}
-
-// Site index of a pair's lane x and the step from it to lane y (the pairing of load_pairs).
-template <int PARITY>
-__device__ __forceinline__ uint32_t pair_site0(const Addr2 &ad) {
-  return (uint32_t)(PARITY == 0 ? ad.s0 : ad.s0 + 1);
-}
-template <int PARITY>
-__device__ __forceinline__ uint32_t pair_dsite(const Addr2 &ad) {
-  return PARITY == 0 ? 1u : (uint32_t)(ad.sp2 - ad.s0 - 1);
-}
 
 // Raw moments of the deviation tile and rho, u (Eq. macro); entry (0,0,0) stays rho - rho0.
 template <int D, typename T>
@@ -575,7 +339,7 @@ __device__ __forceinline__ void iso_rotate(T &a, T &b, T &c) {  // (k4, k5, k6) 
   b = d1;
   c = d2;
 }
-// iso_unrotate, each output halved (the halved convention of the inverse transforms).
+// The inverse of iso_rotate, each output halved (the halved convention of the inverse transforms).
 template <typename T>
 __device__ __forceinline__ void iso_unrotate_h(T &a, T &b, T &c) {
   const T s4 = vmul(splat<T>(1.0f / 12.0f), vfma(splat<T>(2.0f), a, c));  // (k4 + k5) / 4
@@ -586,16 +350,4 @@ __device__ __forceinline__ void iso_unrotate_h(T &a, T &b, T &c) {
   b = k5;
   c = k6;
 }
-template <typename T>
-__device__ __forceinline__ void iso_unrotate(T &a, T &b, T &c) {  // (M4', M5', M6') -> (k4, k5, k6)
-  const T third = splat<T>(1.0f / 3.0f), half = splat<T>(0.5f);
-  const T s = vmul(third, vfma(splat<T>(2.0f), a, c));  // k4 + k5 = (2 M4' + M6') / 3
-  const T k6 = vmul(third, vsub(a, c));                 // (M4' - M6') / 3
-  const T k4 = vmul(half, vadd(s, b));
-  const T k5 = vmul(half, vsub(s, b));
-  a = k4;
-  b = k5;
-  c = k6;
-}
-
 }  // namespace flbm

@@ -3,16 +3,13 @@
 //
 // Velocities are the first 19 of the D3Q27 order (Lat<3>: rest, axes, face diagonals), so
 // population i of D3Q19 is plane i of a 19-plane array, addressed exactly as D3Q27 with
-// the eight corners left out. The moment transforms are the generated straight-line code
-// of d3q19_gen.cuh (raw moments, central shift N(u), its inverse by forward substitution,
-// populations from raw moments); the collision is Eq. cm_collision with k^eq = (rho, 0,
+// the eight corners left out. The collision is Eq. cm_collision with k^eq = (rho, 0,
 // ...), phi_v = sqrt(rho) phc_v and the noisy modes v = 4..18 fed by Philox blocks
 // (v - 4) / 4, slot (v - 4) mod 4, as for the other lattices.
 #pragma once
 
 #include "cm.cuh"
 #include "collide.cuh"
-#include "d3q19_gen.cuh"
 #include "philox.cuh"
 
 namespace flbm {
@@ -54,129 +51,209 @@ __device__ __forceinline__ void store19(S *__restrict__ f, long long plane, cons
       }
 }
 
-template <typename S, int PARITY>
-__device__ __forceinline__ void load19_2(const S *__restrict__ f, long long plane, const Addr2 &ad,
-                                         float2 (&F)[19]) {
-#pragma unroll
-  for (int dz = -1; dz <= 1; ++dz)
-#pragma unroll
-    for (int dy = -1; dy <= 1; ++dy)
-#pragma unroll
-      for (int dx = -1; dx <= 1; ++dx) {
-        if (!d3q19_has(dx, dy, dz)) continue;
-        const int i = Lat<3>::index(dx, dy, dz);
-        float2 v;
-        if (PARITY == 0) {
-          v = Storage2<S>::load(f + i * plane + ad.s0);
-        } else {
-          const S *b = f + opposite<3>(i) * plane + ad.dy[1 - dy] + ad.dz[1 - dz];
-          if (dx == 0) {
-            v = Storage2<S>::load(b + ad.s0);
-          } else if (dx == 1) {
-            v.x = Storage<S>::load(b + ad.sm1);
-            v.y = Storage<S>::load(b + ad.s0);
-          } else {
-            v.x = Storage<S>::load(b + ad.s0 + 1);
-            v.y = Storage<S>::load(b + ad.sp2);
-          }
-        }
-        F[i] = v;
-      }
-}
+// ---- the algebra ---------------------------------------------------------------------------
+// The basis printed in Sec. II-C is not a product of 1-D polynomials, but the 19 products H_abc of
+// 1, c and c^2 - 1/3 with at most two nonzero orders (a, b, c along x, y, z) are a basis of the functions
+// on these velocities. Along an axis they shift as on D3Q27 (cm.cuh), on the five lines that
+// hold all three orders, because lowering an order stays in the set. The paper's modes are
+// combinations of the same products of the shifted velocity, but for third and fourth powers along
+// one axis, which close on the lattice: with c^3 = c,
+//   sum (c_x - u)^3 f = -u (u^2 rho + 3 H_200),
+//   sum (c_x - u)^4 f = rho / 3 + H_200 + E_x,  E_x = u^2 (6 H_200 + rho (3 u^2 - 1)).
+// The lattice's weights have no H but H_000, so the moments of the deviations d_i = f_i - w_i rho0
+// differ from those of f_i in H_000 alone: rho in the shifts, rho - rho0 in the populations.
+// The noisy step was bound by the FMA pipe with N(u) = T(u) M^-1 written out (114 polynomial entries,
+// some 300 operations each way against 150 to 170 here); with the paper's rates it now streams at
+// 0.97 of the measured copy. us per step at 256^3, before -> now: FP32 444 -> 391, BF16 452 -> 371, general
+// rates 507 -> 424, without noise 374 -> 368; statistics 360 -> 311 (even), 393 -> 334 (odd).
 
-template <typename S, int PARITY>
-__device__ __forceinline__ void store19_2(S *__restrict__ f, long long plane, const Addr2 &ad,
-                                          const float2 (&F)[19]) {
-#pragma unroll
-  for (int dz = -1; dz <= 1; ++dz)
-#pragma unroll
-    for (int dy = -1; dy <= 1; ++dy)
-#pragma unroll
-      for (int dx = -1; dx <= 1; ++dx) {
-        if (!d3q19_has(dx, dy, dz)) continue;
-        const int i = Lat<3>::index(dx, dy, dz);
-        const float2 v = F[i];
-        if (PARITY == 0) {
-          Storage2<S>::store(f + opposite<3>(i) * plane + ad.s0, v);
-        } else {
-          S *b = f + i * plane + ad.dy[1 + dy] + ad.dz[1 + dz];
-          if (dx == 0) {
-            Storage2<S>::store(b + ad.s0, v);
-          } else if (dx == 1) {
-            Storage<S>::store(b + ad.s0 + 1, v.x);
-            Storage<S>::store(b + ad.sp2, v.y);
-          } else {
-            Storage<S>::store(b + ad.sm1, v.x);
-            Storage<S>::store(b + ad.s0, v.y);
-          }
-        }
-      }
-}
-
-// The pairing of load_pairs / store_pairs (cm.cuh): on odd steps lanes hold x0 + 1 and x0 + 2,
-// so the populations with c_x = +-1 (10 of 19) move as aligned pairs.
-template <typename S, int PARITY>
-__device__ __forceinline__ void load19_pairs(const S *__restrict__ f, long long plane, const Addr2 &ad,
-                                             float2 (&F)[19]) {
-  if (PARITY == 0) {
-    load19_2<S, 0>(f, plane, ad, F);
-    return;
-  }
-#pragma unroll
-  for (int dz = -1; dz <= 1; ++dz)
-#pragma unroll
-    for (int dy = -1; dy <= 1; ++dy)
-#pragma unroll
-      for (int dx = -1; dx <= 1; ++dx) {
-        if (!d3q19_has(dx, dy, dz)) continue;
-        const int i = Lat<3>::index(dx, dy, dz);
-        const S *b = f + opposite<3>(i) * plane + ad.dy[1 - dy] + ad.dz[1 - dz];
-        float2 v;
-        if (dx == 0) {
-          v.x = Storage<S>::load(b + ad.s0 + 1);
-          v.y = Storage<S>::load(b + ad.sp2);
-        } else {
-          v = Storage2<S>::load(b + (dx == 1 ? ad.s0 : ad.sp2));
-        }
-        F[i] = v;
-      }
-}
-template <typename S, int PARITY>
-__device__ __forceinline__ void store19_pairs(S *__restrict__ f, long long plane, const Addr2 &ad,
-                                              const float2 (&F)[19]) {
-  if (PARITY == 0) {
-    store19_2<S, 0>(f, plane, ad, F);
-    return;
-  }
-#pragma unroll
-  for (int dz = -1; dz <= 1; ++dz)
-#pragma unroll
-    for (int dy = -1; dy <= 1; ++dy)
-#pragma unroll
-      for (int dx = -1; dx <= 1; ++dx) {
-        if (!d3q19_has(dx, dy, dz)) continue;
-        const int i = Lat<3>::index(dx, dy, dz);
-        S *b = f + i * plane + ad.dy[1 + dy] + ad.dz[1 + dz];
-        const float2 v = F[i];
-        if (dx == 0) {
-          Storage<S>::store(b + ad.s0 + 1, v.x);
-          Storage<S>::store(b + ad.sp2, v.y);
-        } else {
-          Storage2<S>::store(b + (dx == 1 ? ad.sp2 : ad.s0), v);
-        }
-      }
-}
-
-// rho, u and the raw moments of the deviations (r_0 = rho - rho0).
+// A face's four diagonals f(+,+), f(-,+), f(+,-), f(-,-): sum, first moments, mixed moment, which are
+// the lattice's second-order products in its plane: a^2 b^2, a b^2, a^2 b and a b.
 template <typename T>
-__device__ __forceinline__ void d3q19_macros(const T (&F)[19], float rho0, T (&r)[19], T &rho, T &ux, T &uy,
-                                             T &uz) {
-  d3q19_raw(F, r);
-  rho = vadd(splat<T>(rho0), r[0]);
-  const T inv_rho = rcp_fast_lanes(rho);
-  ux = vmul(r[1], inv_rho);
-  uy = vmul(r[2], inv_rho);
-  uz = vmul(r[3], inv_rho);
+__device__ __forceinline__ void d3q19_face(const T (&F)[19], int i, T &s, T &da, T &db, T &m) {
+  const T s1 = vadd(F[i], F[i + 1]), s2 = vadd(F[i + 2], F[i + 3]);
+  const T d1 = vsub(F[i], F[i + 1]), d2 = vsub(F[i + 2], F[i + 3]);
+  s = vadd(s1, s2);
+  da = vadd(d1, d2);
+  db = vsub(s1, s2);
+  m = vsub(d1, d2);
+}
+
+// Raw moments of the deviations: drho, j, the mixed second moments P = (xy, yz, xz), the sums a on the
+// axes and the faces' sums s = (xy, yz, xz) and third moments o = (xyy, xzz, yzz, xxy, xxz, yyz).
+template <typename T>
+struct D3Q19Raw {
+  T drho, j[3], P[3], a[3], s[3], o[6];
+  __device__ __forceinline__ explicit D3Q19Raw(const T (&F)[19]) {
+    d3q19_face(F, 7, s[0], o[0], o[3], P[0]);
+    d3q19_face(F, 11, s[2], o[1], o[4], P[2]);
+    d3q19_face(F, 15, s[1], o[2], o[5], P[1]);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) a[k] = vadd(F[1 + 2 * k], F[2 + 2 * k]);
+    drho = vadd(vadd(vadd(F[0], a[0]), vadd(a[1], a[2])), vadd(vadd(s[0], s[2]), s[1]));
+    j[0] = vadd(vsub(F[1], F[2]), vadd(o[0], o[1]));
+    j[1] = vadd(vsub(F[3], F[4]), vadd(o[3], o[2]));
+    j[2] = vadd(vsub(F[5], F[6]), vadd(o[4], o[5]));
+  }
+};
+
+// Central moments k[v - 4] = k_v, v = 4..18, from the raw moments about u = j / rho.
+template <typename T>
+__device__ __forceinline__ void d3q19_central(const D3Q19Raw<T> &r, T rho, const T (&u)[3], T (&k)[15]) {
+  const auto c = [](double x) { return rat<T>(x); };
+  const T third = c(-1.0 / 3.0);
+  T H[3], nu[3];
+  const T M[3] = {vadd(r.a[0], vadd(r.s[0], r.s[2])), vadd(r.a[1], vadd(r.s[0], r.s[1])),
+                  vadd(r.a[2], vadd(r.s[2], r.s[1]))};
+  const T ninth = vmul(c(1.0 / 9.0), r.drho);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    H[a] = vfma(third, r.drho, M[a]);
+    nu[a] = vmul(c(-1.0), u[a]);
+  }
+  T xy = r.P[0], yz = r.P[1], xz = r.P[2];
+  T xyy = vfma(third, r.j[0], r.o[0]), xzz = vfma(third, r.j[0], r.o[1]), yzz = vfma(third, r.j[1], r.o[2]);
+  T xxy = vfma(third, r.j[1], r.o[3]), xxz = vfma(third, r.j[2], r.o[4]), yyz = vfma(third, r.j[2], r.o[5]);
+  T xxyy = vadd(vfma(third, vadd(M[0], M[1]), r.s[0]), ninth);
+  T xxzz = vadd(vfma(third, vadd(M[0], M[2]), r.s[2]), ninth);
+  T yyzz = vadd(vfma(third, vadd(M[1], M[2]), r.s[1]), ninth);
+  // Shifts: the line through H_000 has k_1 = 0 and k_2 = m_2 - u j; a line whose order 0 is a first
+  // moment shifted before starts at zero.
+  T m = r.j[1], n = r.j[2];
+  H[0] = vfma(nu[0], r.j[0], H[0]);  // x: lines (0,0), (1,0), (0,1), (2,0), (0,2) in the orders of (y, z)
+  shift_fwd(m, xy, xxy, nu[0]);
+  shift_fwd(n, xz, xxz, nu[0]);
+  shift_fwd(H[1], xyy, xxyy, nu[0]);
+  shift_fwd(H[2], xzz, xxzz, nu[0]);
+  H[1] = vfma(nu[1], r.j[1], H[1]);  // y: lines (0,0), (1,0), (0,1), (2,0), (0,2) in (x, z)
+  xyy = vfma(nu[1], vadd(xy, xy), xyy);
+  shift_fwd(n, yz, yyz, nu[1]);
+  shift_fwd(H[0], xxy, xxyy, nu[1]);
+  shift_fwd(H[2], yzz, yyzz, nu[1]);
+  H[2] = vfma(nu[2], r.j[2], H[2]);  // z: lines (0,0), (1,0), (0,1), (2,0), (0,2) in (x, y)
+  xzz = vfma(nu[2], vadd(xz, xz), xzz);
+  yzz = vfma(nu[2], vadd(yz, yz), yzz);
+  shift_fwd(H[0], xxz, xxzz, nu[2]);
+  shift_fwd(H[1], yyz, yyzz, nu[2]);
+  // The paper's modes.
+  T E[3], q[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const T u2 = vmul(u[a], u[a]), h3 = vmul(c(3.0), H[a]);
+    q[a] = vmul(u[a], vfma(u2, rho, h3));  // less the cube
+    E[a] = vmul(u2, vfma(c(2.0), h3, vmul(rho, vfma(c(3.0), u2, c(-1.0)))));
+  }
+  k[0] = vadd(H[0], vadd(H[1], H[2]));
+  k[1] = vfma(c(3.0), H[0], vmul(c(-1.0), k[0]));
+  k[2] = vsub(H[1], H[2]);
+  k[3] = xy;
+  k[4] = yz;
+  k[5] = xz;
+  k[6] = vmul(c(3.0), vsub(vadd(xyy, xzz), q[0]));
+  k[7] = vmul(c(3.0), vsub(vadd(xxy, yzz), q[1]));
+  k[8] = vmul(c(3.0), vsub(vadd(xxz, yyz), q[2]));
+  k[9] = vsub(xyy, xzz);
+  k[10] = vsub(yzz, xxy);
+  k[11] = vsub(xxz, yyz);
+  const T A = vadd(xxyy, xxzz), B = vsub(xxyy, xxzz);
+  const T d16 = vfma(c(3.0), vadd(E[0], vadd(E[1], E[2])), vmul(c(6.0), vadd(A, yyzz)));  // k_16 - k_4
+  k[12] = vadd(d16, k[0]);
+  k[13] = vfma(c(6.0), vadd(A, E[0]), vfma(c(-2.0 / 3.0), d16, vmul(third, k[1])));
+  k[14] = vfma(c(2.0), vadd(B, vsub(E[1], E[2])), vmul(third, k[2]));
+}
+
+// Populations (deviations) from the post-collision central moments: k_0 = rho, k_1..3 = 0,
+// k[v - 4] = k_v, and the momentum j = rho u: the 15 definitions solved for the H, the shifts back,
+// and the H in the populations. Throughout, a moment with n nonzero orders is held times 2^-n (the
+// halved convention of cm.cuh).
+template <typename T>
+__device__ __forceinline__ void d3q19_populations(const T (&k)[15], T rho, T drho, const T (&j)[3], const T (&u)[3],
+                                                  T (&F)[19]) {
+  const auto c = [](double x) { return rat<T>(x); };
+  // Second order: H[a] = (H_200, H_020, H_002) / 2 from the trace k_4 and the deviators k_5, k_6.
+  T H[3], xy = vmul(c(0.25), k[3]), yz = vmul(c(0.25), k[4]), xz = vmul(c(0.25), k[5]);
+  H[0] = vmul(c(1.0 / 6.0), vadd(k[0], k[1]));
+  const T rest = vfma(c(-2.0), H[0], k[0]);
+  H[1] = vmul(c(0.25), vadd(rest, k[2]));
+  H[2] = vmul(c(0.25), vsub(rest, k[2]));
+  T E[3], q[3], hu[3], hj[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const T u2 = vmul(u[a], u[a]), h3 = vmul(c(6.0), H[a]);
+    q[a] = vfma(u[a], vfma(u2, rho, h3), vmul(c(1.0 / 3.0), k[6 + a]));  // k_10 / 3 less the cube
+    E[a] = vmul(u2, vfma(c(2.0), h3, vmul(rho, vfma(c(3.0), u2, c(-1.0)))));
+    hu[a] = vmul(c(0.5), u[a]);
+    hj[a] = vmul(c(0.5), j[a]);
+  }
+  // Third order: q_x = H_120 + H_102 and k_13 = H_120 - H_102, and cyclic.
+  const T e8 = c(0.125);
+  T xyy = vmul(e8, vadd(q[0], k[9])), xzz = vmul(e8, vsub(q[0], k[9]));
+  T yzz = vmul(e8, vadd(q[1], k[10])), xxy = vmul(e8, vsub(q[1], k[10]));
+  T xxz = vmul(e8, vadd(q[2], k[11])), yyz = vmul(e8, vsub(q[2], k[11]));
+  // Fourth order: the sum of the three, A = H_220 + H_202 and B = H_220 - H_202.
+  const T d16 = vsub(k[12], k[0]);
+  const T sum = vfma(c(-0.5), vadd(E[0], vadd(E[1], E[2])), vmul(c(1.0 / 6.0), d16));
+  const T A = vfma(c(1.0 / 6.0), k[13], vfma(c(1.0 / 9.0), d16, vfma(c(1.0 / 18.0), k[1], vmul(c(-1.0), E[0]))));
+  const T B = vfma(c(0.5), k[14], vfma(c(1.0 / 6.0), k[2], vsub(E[2], E[1])));
+  T xxyy = vmul(e8, vadd(A, B)), xxzz = vmul(e8, vsub(A, B)), yyzz = vmul(c(0.25), vsub(sum, A));
+  // Shifts. On the line through H_000 the first order is zero and becomes rho u = j; on a line that
+  // starts at a first-order moment still to be shifted (zero) only the second order changes.
+  const auto second = [](T &m2, T h, T v) { m2 = vfma(h, v, m2); };
+  T m = hj[2], n = hj[1];
+  second(H[2], hu[2], j[2]);  // z: lines (0,0), (1,0), (0,1), (2,0), (0,2) in the orders of (x, y)
+  second(xzz, u[2], vadd(xz, xz));
+  second(yzz, u[2], vadd(yz, yz));
+  shift_inv_h(H[0], xxz, xxzz, u[2], hu[2]);
+  shift_inv_h(H[1], yyz, yyzz, u[2], hu[2]);
+  second(H[1], hu[1], j[1]);  // y: lines (0,0), (1,0), (0,1), (2,0), (0,2) in (x, z)
+  second(xyy, u[1], vadd(xy, xy));
+  shift_inv_h(m, yz, yyz, u[1], hu[1]);
+  shift_inv_h(H[0], xxy, xxyy, u[1], hu[1]);
+  shift_inv_h(H[2], yzz, yyzz, u[1], hu[1]);
+  second(H[0], hu[0], j[0]);  // x: lines (0,0), (1,0), (0,1), (2,0), (0,2) in (y, z)
+  shift_inv_h(n, xy, xxy, u[0], hu[0]);
+  shift_inv_h(m, xz, xxz, u[0], hu[0]);
+  shift_inv_h(H[1], xyy, xxyy, u[0], hu[0]);
+  shift_inv_h(H[2], xzz, xxzz, u[0], hu[0]);
+  // Populations, from the monomials (x^2 = H_200 + drho / 3, x y^2 = H_120 + j_x / 3, x^2 y^2 = H_220 +
+  // (H_200 + H_020) / 3 + drho / 9): a face's four diagonals, then what is left on the axes and at rest.
+  T t[3], g[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    t[a] = vfma(c(1.0 / 6.0), H[a], vmul(c(1.0 / 72.0), drho));
+    g[a] = vmul(c(1.0 / 6.0), hj[a]);
+  }
+  xxyy = vadd(xxyy, vadd(t[0], t[1]));
+  xxzz = vadd(xxzz, vadd(t[0], t[2]));
+  yyzz = vadd(yyzz, vadd(t[1], t[2]));
+  xyy = vadd(xyy, g[0]);
+  xzz = vadd(xzz, g[0]);
+  xxy = vadd(xxy, g[1]);
+  yzz = vadd(yzz, g[1]);
+  xxz = vadd(xxz, g[2]);
+  yyz = vadd(yyz, g[2]);
+  const auto face = [&](int i, T even, T odd_a, T odd_b, T mixed) {
+    const T p = vadd(even, mixed), r = vsub(even, mixed);
+    const T s = vadd(odd_a, odd_b), d = vsub(odd_a, odd_b);
+    F[i] = vadd(p, s);
+    F[i + 1] = vsub(r, d);
+    F[i + 2] = vadd(r, d);
+    F[i + 3] = vsub(p, s);
+  };
+  face(7, xxyy, xyy, xxy, xy);
+  face(11, xxzz, xzz, xxz, xz);
+  face(15, yyzz, yzz, yyz, yz);
+  const auto axis = [&](int i, T h2, T e1, T e2, T half_j, T o1, T o2) {
+    const T even = vfma(c(-2.0), vadd(e1, e2), vfma(c(1.0 / 6.0), drho, h2));
+    const T odd = vfma(c(-2.0), vadd(o1, o2), half_j);
+    F[i] = vadd(even, odd);
+    F[i + 1] = vsub(even, odd);
+    return even;
+  };
+  const T ex = axis(1, H[0], xxyy, xxzz, hj[0], xyy, xzz);
+  const T ey = axis(3, H[1], xxyy, yyzz, hj[1], xxy, yzz);
+  const T ez = axis(5, H[2], xxzz, yyzz, hj[2], xxz, yyz);
+  F[0] = vfma(c(-2.0), vfma(c(2.0), vadd(vadd(xxyy, xxzz), yyzz), vadd(vadd(ex, ey), ez)), drho);
 }
 
 // The collision of one site (float) or two (float2); on return F holds the post-collision
@@ -185,33 +262,26 @@ __device__ __forceinline__ void d3q19_macros(const T (&F)[19], float rho0, T (&r
 template <bool NOISE, typename T, bool SHEAR>
 __device__ __forceinline__ void collide19(T (&F)[19], float rho0, const ArrayRates &rates,
                                           const T (&n)[Noisy<19>::count]) {
-  T r[19], rho, ux, uy, uz;
-  d3q19_macros(F, rho0, r, rho, ux, uy, uz);
-  const T jx = r[1], jy = r[2], jz = r[3], drho = r[0];
+  const D3Q19Raw<T> r(F);
+  const T rho = vadd(splat<T>(rho0), r.drho), inv_rho = rcp_fast_lanes(rho);
   const T srho = NOISE ? noise_scale<SHEAR>(rho, rates) : rho;
-  if (SHEAR) {
-    T k[3];
-    d3q19_shear_central(r, rho, ux, uy, uz, k[0], k[1], k[2]);
+  T u[3], k[15];
 #pragma unroll
-    for (int v = 4; v < 19; ++v) r[v] = NOISE ? vmul(srho, n[v - 4]) : splat<T>(0.0f);
+  for (int a = 0; a < 3; ++a) u[a] = vmul(r.j[a], inv_rho);
+  if (SHEAR) {
+#pragma unroll
+    for (int v = 4; v < 19; ++v) k[v - 4] = NOISE ? vmul(srho, n[v - 4]) : splat<T>(0.0f);
+    const int first[3] = {0, 1, 0}, second[3] = {1, 2, 2};  // k_7 (xy), k_8 (yz), k_9 (xz)
 #pragma unroll
     for (int v = 7; v < 10; ++v)
-      r[v] = relaxed<NOISE>(NOISE ? vmul(splat<T>(rates.amp(v)), srho) : srho, n[v - 4], rates.om(v), k[v - 7]);
+      k[v - 4] = relaxed<NOISE>(NOISE ? vmul(splat<T>(rates.amp(v)), srho) : srho, n[v - 4], rates.om(v),
+                                vfma(vmul(splat<T>(-1.0f), r.j[first[v - 7]]), u[second[v - 7]], r.P[v - 7]));
   } else {
-    d3q19_central_lr(r, rho, ux, uy, uz);
+    d3q19_central(r, rho, u, k);
 #pragma unroll
-    for (int v = 4; v < 19; ++v) r[v] = relaxed<NOISE>(srho, n[v - 4], rates.om(v), r[v]);
+    for (int v = 4; v < 19; ++v) k[v - 4] = relaxed<NOISE>(srho, n[v - 4], rates.om(v), k[v - 4]);
   }
-  // The general rates keep more values live; they use the register-lean inverse.
-  if (SHEAR)
-    d3q19_raw_from_central(r, rho, ux, uy, uz);
-  else
-    d3q19_raw_from_central_lr(r, rho, ux, uy, uz);
-  r[0] = drho;  // populations as deviations from w rho0
-  r[1] = jx;    // r*_a = j_a (momentum conserved)
-  r[2] = jy;
-  r[3] = jz;
-  d3q19_pop(r, F);
+  d3q19_populations(k, rho, r.drho, r.j, u, F);
 }
 
 }  // namespace flbm

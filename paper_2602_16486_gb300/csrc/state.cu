@@ -6,11 +6,11 @@
 //   f^eq_i = rho * prod_a g(c_ia, u_a),  g(0, u) = 2/3 - u^2,  g(+-1, u) = (1 +- 3u + 3u^2)/6,
 // which is what the initialiser evaluates (FP64, once per run). D3Q19 (lattice code 19)
 // has no product form; its equilibrium is the state with central moments (rho, 0, ..., 0),
-// built in FP64 with the generated transforms of d3q19_gen.cuh.
+// built in FP64 by d3q19_populations.
 #include <cuda_runtime.h>
 
 #include "cm.cuh"
-#include "d3q19_gen.cuh"
+#include "d3q19.cuh"
 #include "internal.h"
 #include "philox.cuh"
 
@@ -49,17 +49,12 @@ __global__ void init_kernel(S *__restrict__ f, long long plane, int nx, int ny, 
   }
   constexpr int Q = Lat<D>::Q;
   if constexpr (D == 19) {
-    // r* from k^eq = (rho, 0, ...): rows 4..18 by the inverse shift, r*_0 = rho - rho0,
-    // r*_a = rho u_a; then the deviations M^{-1} r*.
-    double r[19], d[19];
+    // k^eq = (rho, 0, ..., 0) at velocity u.
+    double k[15], d[19];
 #pragma unroll
-    for (int v = 0; v < 19; ++v) r[v] = 0.0;
-    d3q19_raw_from_central(r, rho, ux, uy, uz);
-    r[0] = rho - rho0;
-    r[1] = rho * ux;
-    r[2] = rho * uy;
-    r[3] = rho * uz;
-    d3q19_pop(r, d);
+    for (int v = 0; v < 15; ++v) k[v] = 0.0;
+    const double j[3] = {rho * ux, rho * uy, rho * uz}, u[3] = {ux, uy, uz};
+    d3q19_populations(k, rho, rho - rho0, j, u, d);
 #pragma unroll
     for (int i = 0; i < 19; ++i) Storage<S>::store(f + (long long)i * plane + s, (float)d[i]);
   } else {

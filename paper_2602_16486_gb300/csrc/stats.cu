@@ -82,25 +82,25 @@ __device__ __forceinline__ void load_pair(const StepArgs &a, uint32_t k, PairPop
 }
 
 // The columns of the pair from its populations. D3Q19: [1, rho - rho0, j, u, k_4 .. k_18,
-// 0 ...] from the generated transforms of d3q19_gen.cuh; D2Q9 / D3Q27: gram::moment_columns.
+// 0 ...] (d3q19.cuh); D2Q9 / D3Q27: gram::moment_columns.
 template <int D, bool ISO>
 __device__ __forceinline__ void pair_columns(PairPops<D> &P, float rho0, bool v0, bool v1,
                                              float2 (&col)[StatsPlan<D>::NC], unsigned &nonfinite) {
   if constexpr (D == 19) {
-    float2 r[19], rho, ux, uy, uz;
-    d3q19_macros(P.F, rho0, r, rho, ux, uy, uz);
-    const float2 drho = r[0];
-    d3q19_central(r, rho, ux, uy, uz);
-    col[0] = make_float2(v0 ? 1.0f : 0.0f, v1 ? 1.0f : 0.0f);
-    col[1] = drho;
-    col[2] = vmul(rho, ux);
-    col[3] = vmul(rho, uy);
-    col[4] = vmul(rho, uz);
-    col[5] = ux;
-    col[6] = uy;
-    col[7] = uz;
+    const D3Q19Raw<float2> r(P.F);
+    const float2 rho = vadd(splat<float2>(rho0), r.drho), inv_rho = rcp_fast_lanes(rho);
+    float2 u[3], k[15];
 #pragma unroll
-    for (int v = 4; v < 19; ++v) col[8 + v - 4] = r[v];
+    for (int a = 0; a < 3; ++a) {
+      u[a] = vmul(r.j[a], inv_rho);
+      col[2 + a] = vmul(rho, u[a]);
+      col[5 + a] = u[a];
+    }
+    d3q19_central(r, rho, u, k);
+    col[0] = make_float2(v0 ? 1.0f : 0.0f, v1 ? 1.0f : 0.0f);
+    col[1] = r.drho;
+#pragma unroll
+    for (int v = 4; v < 19; ++v) col[8 + v - 4] = k[v - 4];
 #pragma unroll
     for (int c = 8 + 15; c < StatsPlan<D>::NC; ++c) col[c] = make_float2(0.0f, 0.0f);
     float2 sum = col[1];
