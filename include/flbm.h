@@ -224,13 +224,16 @@ int flbm_stats_noalloc(int lattice, const int64_t dims[3], int storage, int pari
  * update): 0 = default (chosen by size, storage and noise), 1 = one site per thread, 2..8 =
  * two sites per thread with the sites flattened over the rows, so that every row length
  * fills the warps; 2, 3, 4 and 8 form 64-bit offsets, 5, 6 and 7 32-bit ones (a plane of
- * 4 GB or more always takes 64). flbm_get_step_variant reports 0 as 2, every choice as 1
- * when nx is odd (two sites per thread run all the same, unless 1 was chosen), and 4 as 2
- * unless nx is even, at most 512 and a row of populations a multiple of 16 bytes.
+ * 4 GB or more always takes 64). By default and with 7 or 8, a call of many steps (six in
+ * 2-D, ten in 3-D) on a small FP32 box (8192 sites in 2-D, 4096 in 3-D) is one launch.
+ * flbm_get_step_variant reports 0 as 2, every choice as 1 when nx is odd (two sites per
+ * thread run all the same, unless 1 was chosen), and 4 as 2 unless nx is even, at most 512
+ * and a row of populations a multiple of 16 bytes.
  * The environment variable FLBM_STEP_VARIANT, read by flbm_create, sets the initial
  * choice.
- * flbm_autotune times variants 1, 2 and 5 over trial_steps steps on a copy of the current state (restored afterwards: populations
- * and step count are unchanged), keeps the fastest for this context and caches the
+ * flbm_autotune times variants 1, 2 and 5 (and 7 on such a box, each over 20 steps at
+ * least) over trial_steps steps on a copy of the current state (restored afterwards:
+ * populations and step count are unchanged), keeps the fastest for this context and caches the
  * choice per (GPU model, lattice, storage, nx parity, size class, noise on/off, rate
  * structure, collision model, nx < 256) for the process; when the environment variable
  * FLBM_AUTOTUNE_CACHE names a file, choices are also read from it (at the first

@@ -337,6 +337,13 @@ int launch_variant(const flbm_ctx *c) {
   return dram ? int(kStepPair) : int(kStepPairOcc);
 }
 
+// Whether a call of n steps runs as one launch (step_cluster.cu): by default, and for the variants
+// that stood for short rows.
+bool takes_cluster(const flbm_ctx *c, int64_t n) {
+  return (c->variant == kStepAuto || c->variant == kStepPairOccRows || c->variant == kStepPairRows) && !c->slab &&
+         cluster_applies(c->lattice, c->storage, c->N, n);
+}
+
 struct CkptHeader {
   char magic[8];
   int32_t version, lattice, storage, q;  // version 2 adds `model` (version 1: central moments)
@@ -478,6 +485,17 @@ int flbm_step(flbm_ctx *c, int64_t n) {
                              "step taken from an odd step count, see flbm_slab_halo)");
   DeviceGuard g(c->device);
   const bool noise = c->kBT > 0.0;
+  if (takes_cluster(c, n)) {
+    for (int64_t left = n; left > 0;) {
+      const int k = int(left < (1 << 20) ? left : (1 << 20));
+      c->args.step_lo = uint32_t(uint64_t(c->step));
+      c->args.step_hi = uint32_t(uint64_t(c->step) >> 32);
+      FLBM_CUDA(launch_step_cluster(c->lattice, c->model == FLBM_COLLISION_RAW, noise, c->shear, c->args, k, c->stream));
+      c->step += k;
+      left -= k;
+    }
+    return FLBM_OK;
+  }
   for (int64_t s = 0; s < n; ++s) {
     c->args.step_lo = uint32_t(uint64_t(c->step));
     c->args.step_hi = uint32_t(uint64_t(c->step) >> 32);
@@ -797,7 +815,11 @@ int flbm_autotune(flbm_ctx *c, int trial_steps, int *chosen) {
       st = fail(FLBM_ECUDA, "autotune set-up: %s", cudaGetErrorString(cudaGetLastError()));
       break;
     }
-    for (int v : {int(kStepOneSite), int(kStepPair), int(kStepPairOcc)}) {
+    // A small box's calls of many steps run in one launch: tried over enough of them to show it.
+    const bool small = cluster_applies(c->lattice, c->storage, c->N, 20);
+    if (small && trial_steps < 20) trial_steps = 20;
+    for (int v : {int(kStepOneSite), int(kStepPair), int(kStepPairOcc), int(kStepPairOccRows)}) {
+      if (v == kStepPairOccRows && !small) continue;
       c->variant = v;
       if ((st = flbm_step(c, 2)) != FLBM_OK) break;  // warm-up (both parities)
       cudaEventRecord(e0, c->stream);

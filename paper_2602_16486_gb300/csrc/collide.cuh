@@ -121,11 +121,12 @@ __device__ __forceinline__ T noise_scale(T rho, const R &rates) {
   return r;
 }
 
-// om k + s n: the relaxed deviation of a mode from its equilibrium plus its noise.
+// om k + s n: the relaxed deviation of a mode from its equilibrium plus its noise. Rounded on its own
+// without noise too (a packed product may be contracted into the sum that takes it, a scalar
+// one may not, and one site and two per thread are to give the same bits).
 template <bool NOISE, typename T>
 __device__ __forceinline__ T relaxed(T s, T n, float om, T k) {
-  const T r = vmul(splat<T>(om), k);
-  return NOISE ? vfma(s, n, r) : r;
+  return NOISE ? vfma(s, n, vmul(splat<T>(om), k)) : vfma(splat<T>(om), k, splat<T>(0.0f));
 }
 
 // The raw-moment counterpart of the scheme (T = M, N = I; Sec. II-C notes that this

@@ -105,7 +105,7 @@ __device__ __forceinline__ void d3q19_central(const D3Q19Raw<T> &r, T rho, const
   T H[3], nu[3];
   const T M[3] = {vadd(r.a[0], vadd(r.s[0], r.s[2])), vadd(r.a[1], vadd(r.s[0], r.s[1])),
                   vadd(r.a[2], vadd(r.s[2], r.s[1]))};
-  const T ninth = vmul(c(1.0 / 9.0), r.drho);
+  const T ninth = c(1.0 / 9.0);
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     H[a] = vfma(third, r.drho, M[a]);
@@ -114,9 +114,9 @@ __device__ __forceinline__ void d3q19_central(const D3Q19Raw<T> &r, T rho, const
   T xy = r.P[0], yz = r.P[1], xz = r.P[2];
   T xyy = vfma(third, r.j[0], r.o[0]), xzz = vfma(third, r.j[0], r.o[1]), yzz = vfma(third, r.j[1], r.o[2]);
   T xxy = vfma(third, r.j[1], r.o[3]), xxz = vfma(third, r.j[2], r.o[4]), yyz = vfma(third, r.j[2], r.o[5]);
-  T xxyy = vadd(vfma(third, vadd(M[0], M[1]), r.s[0]), ninth);
-  T xxzz = vadd(vfma(third, vadd(M[0], M[2]), r.s[2]), ninth);
-  T yyzz = vadd(vfma(third, vadd(M[1], M[2]), r.s[1]), ninth);
+  T xxyy = vfma(ninth, r.drho, vfma(third, vadd(M[0], M[1]), r.s[0]));
+  T xxzz = vfma(ninth, r.drho, vfma(third, vadd(M[0], M[2]), r.s[2]));
+  T yyzz = vfma(ninth, r.drho, vfma(third, vadd(M[1], M[2]), r.s[1]));
   // Shifts: the line through H_000 has k_1 = 0 and k_2 = m_2 - u j; a line whose order 0 is a first
   // moment shifted before starts at zero.
   T m = r.j[1], n = r.j[2];
@@ -136,12 +136,13 @@ __device__ __forceinline__ void d3q19_central(const D3Q19Raw<T> &r, T rho, const
   shift_fwd(H[0], xxz, xxzz, nu[2]);
   shift_fwd(H[1], yyz, yyzz, nu[2]);
   // The paper's modes.
-  T E[3], q[3];
+  T u2[3], X[3], cube[3];  // E_x = u2 X, the cube -u times `cube`
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    const T u2 = vmul(u[a], u[a]), h3 = vmul(c(3.0), H[a]);
-    q[a] = vmul(u[a], vfma(u2, rho, h3));  // less the cube
-    E[a] = vmul(u2, vfma(c(2.0), h3, vmul(rho, vfma(c(3.0), u2, c(-1.0)))));
+    const T h3 = vmul(c(3.0), H[a]);
+    u2[a] = vmul(u[a], u[a]);
+    cube[a] = vfma(u2[a], rho, h3);
+    X[a] = vfma(c(2.0), h3, vmul(rho, vfma(c(3.0), u2[a], c(-1.0))));
   }
   k[0] = vadd(H[0], vadd(H[1], H[2]));
   k[1] = vfma(c(3.0), H[0], vmul(c(-1.0), k[0]));
@@ -149,23 +150,25 @@ __device__ __forceinline__ void d3q19_central(const D3Q19Raw<T> &r, T rho, const
   k[3] = xy;
   k[4] = yz;
   k[5] = xz;
-  k[6] = vmul(c(3.0), vsub(vadd(xyy, xzz), q[0]));
-  k[7] = vmul(c(3.0), vsub(vadd(xxy, yzz), q[1]));
-  k[8] = vmul(c(3.0), vsub(vadd(xxz, yyz), q[2]));
+  k[6] = vmul(c(3.0), vfma(nu[0], cube[0], vadd(xyy, xzz)));
+  k[7] = vmul(c(3.0), vfma(nu[1], cube[1], vadd(xxy, yzz)));
+  k[8] = vmul(c(3.0), vfma(nu[2], cube[2], vadd(xxz, yyz)));
   k[9] = vsub(xyy, xzz);
   k[10] = vsub(yzz, xxy);
   k[11] = vsub(xxz, yyz);
   const T A = vadd(xxyy, xxzz), B = vsub(xxyy, xxzz);
-  const T d16 = vfma(c(3.0), vadd(E[0], vadd(E[1], E[2])), vmul(c(6.0), vadd(A, yyzz)));  // k_16 - k_4
+  const T E0 = vmul(u2[0], X[0]);
+  const T d16 = vfma(c(3.0), vfma(u2[2], X[2], vfma(u2[1], X[1], E0)), vmul(c(6.0), vadd(A, yyzz)));  // k_16 - k_4
   k[12] = vadd(d16, k[0]);
-  k[13] = vfma(c(6.0), vadd(A, E[0]), vfma(c(-2.0 / 3.0), d16, vmul(third, k[1])));
-  k[14] = vfma(c(2.0), vadd(B, vsub(E[1], E[2])), vmul(third, k[2]));
+  k[13] = vfma(c(6.0), vfma(u2[0], X[0], A), vfma(c(-2.0 / 3.0), d16, vmul(third, k[1])));
+  k[14] = vfma(c(2.0), vfma(vmul(c(-1.0), u2[2]), X[2], vfma(u2[1], X[1], B)), vmul(third, k[2]));
 }
 
 // Populations (deviations) from the post-collision central moments: k_0 = rho, k_1..3 = 0,
 // k[v - 4] = k_v, and the momentum j = rho u: the 15 definitions solved for the H, the shifts back,
 // and the H in the populations. Throughout, a moment with n nonzero orders is held times 2^-n (the
-// halved convention of cm.cuh).
+// halved convention of cm.cuh). Products enter sums by explicit multiply-adds throughout, so that one
+// site and two sites per thread round alike.
 template <typename T>
 __device__ __forceinline__ void d3q19_populations(const T (&k)[15], T rho, T drho, const T (&j)[3], const T (&u)[3],
                                                   T (&F)[19]) {
@@ -176,12 +179,13 @@ __device__ __forceinline__ void d3q19_populations(const T (&k)[15], T rho, T drh
   const T rest = vfma(c(-2.0), H[0], k[0]);
   H[1] = vmul(c(0.25), vadd(rest, k[2]));
   H[2] = vmul(c(0.25), vsub(rest, k[2]));
-  T E[3], q[3], hu[3], hj[3];
+  T u2[3], X[3], q[3], hu[3], hj[3];  // E_x = u2 X
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    const T u2 = vmul(u[a], u[a]), h3 = vmul(c(6.0), H[a]);
-    q[a] = vfma(u[a], vfma(u2, rho, h3), vmul(c(1.0 / 3.0), k[6 + a]));  // k_10 / 3 less the cube
-    E[a] = vmul(u2, vfma(c(2.0), h3, vmul(rho, vfma(c(3.0), u2, c(-1.0)))));
+    const T h3 = vmul(c(6.0), H[a]);
+    u2[a] = vmul(u[a], u[a]);
+    q[a] = vfma(u[a], vfma(u2[a], rho, h3), vmul(c(1.0 / 3.0), k[6 + a]));  // k_10 / 3 less the cube
+    X[a] = vfma(c(2.0), h3, vmul(rho, vfma(c(3.0), u2[a], c(-1.0))));
     hu[a] = vmul(c(0.5), u[a]);
     hj[a] = vmul(c(0.5), j[a]);
   }
@@ -192,9 +196,13 @@ __device__ __forceinline__ void d3q19_populations(const T (&k)[15], T rho, T drh
   T xxz = vmul(e8, vadd(q[2], k[11])), yyz = vmul(e8, vsub(q[2], k[11]));
   // Fourth order: the sum of the three, A = H_220 + H_202 and B = H_220 - H_202.
   const T d16 = vsub(k[12], k[0]);
-  const T sum = vfma(c(-0.5), vadd(E[0], vadd(E[1], E[2])), vmul(c(1.0 / 6.0), d16));
-  const T A = vfma(c(1.0 / 6.0), k[13], vfma(c(1.0 / 9.0), d16, vfma(c(1.0 / 18.0), k[1], vmul(c(-1.0), E[0]))));
-  const T B = vfma(c(0.5), k[14], vfma(c(1.0 / 6.0), k[2], vsub(E[2], E[1])));
+  T m2[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) m2[a] = vmul(c(-1.0), u2[a]);
+  const T mE0 = vmul(m2[0], X[0]);
+  const T sum = vfma(c(0.5), vfma(m2[2], X[2], vfma(m2[1], X[1], mE0)), vmul(c(1.0 / 6.0), d16));
+  const T A = vfma(c(1.0 / 6.0), k[13], vfma(c(1.0 / 9.0), d16, vfma(c(1.0 / 18.0), k[1], mE0)));
+  const T B = vfma(c(0.5), k[14], vfma(c(1.0 / 6.0), k[2], vfma(u2[2], X[2], vmul(m2[1], X[1]))));
   T xxyy = vmul(e8, vadd(A, B)), xxzz = vmul(e8, vsub(A, B)), yyzz = vmul(c(0.25), vsub(sum, A));
   // Shifts. On the line through H_000 the first order is zero and becomes rho u = j; on a line that
   // starts at a first-order moment still to be shifted (zero) only the second order changes.
@@ -217,21 +225,18 @@ __device__ __forceinline__ void d3q19_populations(const T (&k)[15], T rho, T drh
   shift_inv_h(H[2], xzz, xxzz, u[0], hu[0]);
   // Populations, from the monomials (x^2 = H_200 + drho / 3, x y^2 = H_120 + j_x / 3, x^2 y^2 = H_220 +
   // (H_200 + H_020) / 3 + drho / 9): a face's four diagonals, then what is left on the axes and at rest.
-  T t[3], g[3];
+  T t[3];
 #pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    t[a] = vfma(c(1.0 / 6.0), H[a], vmul(c(1.0 / 72.0), drho));
-    g[a] = vmul(c(1.0 / 6.0), hj[a]);
-  }
+  for (int a = 0; a < 3; ++a) t[a] = vfma(c(1.0 / 6.0), H[a], vmul(c(1.0 / 72.0), drho));
   xxyy = vadd(xxyy, vadd(t[0], t[1]));
   xxzz = vadd(xxzz, vadd(t[0], t[2]));
   yyzz = vadd(yyzz, vadd(t[1], t[2]));
-  xyy = vadd(xyy, g[0]);
-  xzz = vadd(xzz, g[0]);
-  xxy = vadd(xxy, g[1]);
-  yzz = vadd(yzz, g[1]);
-  xxz = vadd(xxz, g[2]);
-  yyz = vadd(yyz, g[2]);
+  xyy = vfma(c(1.0 / 6.0), hj[0], xyy);
+  xzz = vfma(c(1.0 / 6.0), hj[0], xzz);
+  xxy = vfma(c(1.0 / 6.0), hj[1], xxy);
+  yzz = vfma(c(1.0 / 6.0), hj[1], yzz);
+  xxz = vfma(c(1.0 / 6.0), hj[2], xxz);
+  yyz = vfma(c(1.0 / 6.0), hj[2], yyz);
   const auto face = [&](int i, T even, T odd_a, T odd_b, T mixed) {
     const T p = vadd(even, mixed), r = vsub(even, mixed);
     const T s = vadd(odd_a, odd_b), d = vsub(odd_a, odd_b);

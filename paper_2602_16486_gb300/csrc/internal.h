@@ -147,6 +147,10 @@ cudaError_t launch_step_d3q19(int storage, int variant, int parity, bool noise, 
 // The raw-moment collision (step_raw.cu): D 2 or 3.
 cudaError_t launch_step_raw(int D, int storage, int variant, int parity, bool noise, const StepArgs &a,
                             cudaStream_t s);
+// nsteps updates of a small FP32 box in one launch (step_cluster.cu), where cluster_applies.
+bool cluster_applies(int lattice, int storage, long long sites, long long nsteps);
+cudaError_t launch_step_cluster(int lattice, bool raw, bool noise, bool shear, const StepArgs &a, int nsteps,
+                                cudaStream_t s);
 // Statistics of the sites a step of `a` would update (the whole box, or a slab's owned planes) to
 // the record `out`; work: stats_record_len zeros, zero again when the launch ends, and a ticket
 // counter likewise; or both null and `out` cleared beforehand.

@@ -132,3 +132,35 @@ def test_batch_lattice_of_4_gb(fl, oracle_mod):
         for step in (0, 1):
             assert _streamed_match_oracle(lat, oracle_mod, 1, dims, _lam(27, "paper"), 1e-4, 4, sites,
                                           lambda: b.step(1), step) <= TOL
+
+
+CLUSTERS = [(0, (1, 1, 1)), (0, (3, 5, 1)), (0, (7, 9, 1)), (0, (33, 17, 1)), (0, (64, 64, 1)), (0, (1, 700, 1)),
+            (0, (91, 90, 1)), (1, (2, 1, 3)), (1, (5, 4, 3)), (1, (16, 16, 16)), (1, (15, 13, 21)), (2, (9, 5, 4)),
+            (3, (7, 6, 5)), (3, (1, 64, 64))]
+
+
+@pytest.mark.parametrize("lattice,dims", CLUSTERS)
+@pytest.mark.parametrize("rates", ["paper", "general", "raw"])
+def test_many_steps_of_a_small_box(fl, oracle_mod, lattice, dims, rates):
+    # One cluster launch for a call's steps (even and odd counts, from either parity) against the
+    # oracle, and bit for bit against the pair kernels stepping once per launch.
+    if rates == "raw" and lattice > 1:
+        pytest.skip("the raw-moment collision is built for D2Q9 and D3Q27")
+    q = (9, 27, 27, 19)[lattice]
+    lam, w = _lam(q, rates), oracle_mod.tables(lattice)[1].reshape(q, 1, 1, 1)
+    for kbt in (1e-4, 0.0):
+        out = []
+        for variant in (0, 5):
+            with fl.Lattice(lattice, dims, lam, kbt, 1.0, (1 << 33) + 7) as lat:
+                lat.variant = variant
+                if rates == "raw":
+                    lat.collision = fl.FLBM_COLLISION_RAW
+                lat.init_uniform((0.04, -0.02, 0.01), 1e-3, 3)
+                f0 = lat.populations()
+                for n in (11, 4, 12, 1, 10):
+                    lat.step(n)
+                assert lat.step_count == 38
+                out.append(lat.populations())
+        fo = oracle_mod.run(lattice, dims, lam, kbt, (1 << 33) + 7, f0, 0, 38, model=int(rates == "raw"))
+        assert (np.abs(out[0] - fo) / w).max() <= TOL, kbt
+        assert np.array_equal(out[0], out[1]), kbt
