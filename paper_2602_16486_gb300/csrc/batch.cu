@@ -13,9 +13,9 @@
 // (pair_kernel, step_kernels.cuh): reads staged by cp.async while the noise is formed, the next
 // launch's blocks starting as this one drains. It is bound like it by the FMA pipe; what a batch
 // adds is the addressing (a lattice's array and plane are not kernel arguments of their own).
-// us per step, before -> now, in the shape the autotuner picks: 32 D3Q27 64^3 321 -> 281, one
-// 256^3 634 -> 568, 233 of 33^3 368 -> 338, 512 of 16^3 86 -> 74, 256 D2Q9 256^2 201 -> 195, 256 of
-// 255^2 228 -> 216; 256 mixed lattices (10.7 M sites) 392 -> 360.
+// us per step, before -> now, in the shape the autotuner picks: 32 D3Q27 64^3 321 -> 277, one
+// 256^3 634 -> 564, 233 of 33^3 368 -> 338, 512 of 16^3 86 -> 72, 256 D2Q9 256^2 201 -> 185, 256 of
+// 255^2 228 -> 210; 256 mixed lattices (10.7 M sites) 392 -> 355.
 //
 // Persistent form: one cooperative launch runs n steps; block b takes the work items
 // (step s, tile b + j G) in step-major order. There is no grid-wide barrier between
@@ -119,9 +119,8 @@ __device__ __forceinline__ void batch_pair(const BatchLattice &L, const Base &pl
     }
   };
   begin(early);
-  lattice_noise<D, SHEAR, 0, B / 2>(n, L, rates, s0, dsite, step);
+  lattice_noise<D, SHEAR, 0, B>(n, L, rates, s0, dsite, step);
   if (!early) begin(true);
-  lattice_noise<D, SHEAR, B / 2, B>(n, L, rates, s0, dsite, step);
   if (STAGE) cp_async_wait_all();
   if (STAGE || aligned)
     pair_of<D, PARITY, true, STAGE, O, THREADS>(L, planes, slot).load_tile(stage, F);

@@ -11,10 +11,12 @@
 namespace flbm {
 
 constexpr int kStepBlock = 128;   // threads per block of the step kernels
-// Pair slots from which a step launch is longer than two rounds of the GPU (152 SMs, five blocks
-// each): its blocks then read before they form any noise, and the launch before it has long
-// drained. Shorter launches overlap noise with that drain instead.
-constexpr uint32_t kEarlySlots = 2u * 152u * 5u * 128u;
+// Pair slots above which a step launch is longer than three rounds of the GPU (152 SMs, five blocks
+// each): its blocks then read before they form the noise. Below, the noise goes before the wait for
+// the step before. us per step, noise first / reads first: D3Q27 64^3 (131 k slots) 9.9 / 10.4, 80^3
+// (256 k) 17.5 / 18.8, 96^3 (442 k) 30.5 / 29.9, 128^3 79.9 / 73.7; D2Q9 512^2 3.5 / 4.2, 1024^2 (524 k)
+// 11.2 / 11.1, 2048^2 48.9 / 46.4.
+constexpr uint32_t kEarlySlots = 3u * 152u * 5u * 128u;
 constexpr int kStatsBlock = 128;  // threads (= sites per tile) of the statistics kernel
 
 // Arguments of one fused step launch (passed by value, lives in the constant bank).
@@ -47,7 +49,7 @@ struct StepArgs {
   float phc_t[27];    // constants the D2Q9 / D3Q27 collision takes (isotropic modes 4-6: 1)
   float amp[27];      // sqrt(Lambda_v (2 - Lambda_v))
   float sqrt_kbt;
-  bool early;         // more blocks than two rounds of the GPU: read before forming any noise
+  bool early;         // a long launch: read before forming any noise (kEarlySlots)
 };
 
 // ---- batched ensembles (batch.cu) ----------------------------------------------------

@@ -83,8 +83,8 @@ __global__ void __launch_bounds__(kStepBlock, MINB) pair_kernel(const StepArgs a
       p.init_row(PlaneTable{a.pop}, x0, y, z + a.z_lo, a.nx, a.ny, a.nz);
     }
   }
-  // Large launches: every read first, all of the noise while the populations travel. Small ones:
-  // half of the noise before the wait for the step before (it fills the drain of that launch).
+  // Large launches: the reads first, the noise while the populations travel. Small ones: the noise
+  // before the wait for the step before, so that it fills the drain of that launch.
   constexpr int B = Noisy<LAT>::blocks;
   float2 n[Noisy<LAT>::count];
   const uint32_t st = shared_address(stage + threadIdx.x);
@@ -92,12 +92,11 @@ __global__ void __launch_bounds__(kStepBlock, MINB) pair_kernel(const StepArgs a
     wait_prerequisites();
     p.fetch(st);
   }
-  if (NOISE) site_noise<LAT, SCHEME, ISO, 0, B / 2>(n, a, p.site0, p.dsite, a.step_lo, a.step_hi);
+  if (NOISE) site_noise<LAT, SCHEME, ISO, 0, B>(n, a, p.site0, p.dsite, a.step_lo, a.step_hi);
   if (!a.early) {
     wait_prerequisites();
     p.fetch(st);
   }
-  if (NOISE) site_noise<LAT, SCHEME, ISO, B / 2, B>(n, a, p.site0, p.dsite, a.step_lo, a.step_hi);
   if (Access::STAGED) cp_async_wait_all();
   if constexpr (LAT == 19) {
     float2 F[19];
