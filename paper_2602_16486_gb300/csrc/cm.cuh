@@ -52,7 +52,7 @@ template <typename T>
 __device__ __forceinline__ void raw_fwd(T &p0, T &p1, T &p2) {
   const T e = vadd(p2, p0);
   const T s = vadd(p1, e);
-  const T d = vsub(p2, p0);
+  const T d = vdiff(p2, p0);
   p2 = vfma(splat<T>(-kCs2), s, e);
   p1 = d;
   p0 = s;
@@ -74,7 +74,7 @@ template <typename T>
 __device__ __forceinline__ void raw_inv_h(T &p0, T &p1, T &p2) {
   const T s = p0;
   const T e = vfma(splat<T>(0.5f * kCs2), s, p2);  // (cs^2 s + p2) / 2
-  p0 = vsub(e, p1);
+  p0 = vdiff(e, p1);
   p2 = vadd(e, p1);
   p1 = vfma(splat<T>(-2.0f), e, s);
 }
@@ -127,30 +127,80 @@ __device__ __forceinline__ void tile_shift_fwd(T (&F)[3][3][3], T nux, T nuy, T 
   }
 }
 
-// Inverses of the whole tile in the halved convention (tile_scale in lattice.cuh): central
-// moments scaled by 2^-(nonzero orders) -> raw moments (same scaling) -> populations.
+// Inverse of a tile of central moments in the halved convention (tile_scale in lattice.cuh: every
+// entry scaled by 2^-(nonzero orders)) to the deviations of the populations, with the zeroth moment
+// rho (rho - rho0 = drho once it is raw) and first central moments of zero; these four entries are
+// not read, and lines that start from a zero take one operation for their shift, k2 + 2u k1. Shifts along z and y, then the shift and the raw inverse of the x axis in one, then
+// the raw inverses along y and z: the axes' transforms commute, and rho turns into drho between
+// the shifts and the raw inverses, which is one line of the joint pass. Joint, a line takes 6
+// operations instead of 7:
+//   e = k2/2 + 2u (k1/2) + (u^2 + cs^2) k0 / 2,  r1/2 = k1/2 + u k0 / 2,  v(+-1) = e +- r1/2,  v(0) = k0 - 2e.
 template <int D, typename T>
-__device__ __forceinline__ void tile_shift_inv_h(T (&F)[3][3][3], T ux, T uy, T uz) {
+__device__ __forceinline__ void tile_inv_h(T (&F)[3][3][3], T rho, T drho, T ux, T uy, T uz) {
   constexpr int z0 = (D == 3) ? 0 : 1, z1 = (D == 3) ? 3 : 2;
-  const T h = splat<T>(0.5f);
+  const T h = splat<T>(0.5f), zero = splat<T>(0.0f);
   if (D == 3) {
-    const T huz = vmul(h, uz);
+    const T huz = vmul(h, uz), tuz = vmul(splat<T>(2.0f), uz);
 #pragma unroll
     for (int b = 0; b < 3; ++b)
 #pragma unroll
-      for (int a = 0; a < 3; ++a) shift_inv_h(F[0][b][a], F[1][b][a], F[2][b][a], uz, huz);
+      for (int a = 0; a < 3; ++a) {
+        if (a + b == 0) {
+          F[1][0][0] = vfma(huz, rho, zero);
+          F[2][0][0] = vfma(uz, F[1][0][0], F[2][0][0]);
+        } else if (a + b == 1) {
+          F[2][b][a] = vfma(tuz, F[1][b][a], F[2][b][a]);
+        } else {
+          shift_inv_h(F[0][b][a], F[1][b][a], F[2][b][a], uz, huz);
+        }
+      }
   }
-  const T huy = vmul(h, uy), hux = vmul(h, ux);
+  const T huy = vmul(h, uy), hux = vmul(h, ux), tuy = vmul(splat<T>(2.0f), uy);
 #pragma unroll
   for (int z = z0; z < z1; ++z)
 #pragma unroll
-    for (int a = 0; a < 3; ++a) shift_inv_h(F[z][0][a], F[z][1][a], F[z][2][a], uy, huy);
+    for (int a = 0; a < 3; ++a) {
+      if (z == z0 && a == 0) {
+        F[z][1][0] = vfma(huy, rho, zero);
+        F[z][2][0] = vfma(uy, F[z][1][0], F[z][2][0]);
+      } else if (z == z0 && a == 1) {
+        F[z][2][1] = vfma(tuy, F[z][1][1], F[z][2][1]);
+      } else {
+        shift_inv_h(F[z][0][a], F[z][1][a], F[z][2][a], uy, huy);
+      }
+    }
+  const T tux = vmul(splat<T>(2.0f), ux), al = vfma(ux, hux, splat<T>(0.5f * kCs2));
 #pragma unroll
   for (int z = z0; z < z1; ++z)
 #pragma unroll
-    for (int b = 0; b < 3; ++b) shift_inv_h(F[z][b][0], F[z][b][1], F[z][b][2], ux, hux);
+    for (int b = 0; b < 3; ++b) {
+      T s, e, r;
+      if (z == z0 && b == 0) {
+        s = drho;
+        r = vfma(hux, rho, zero);
+        e = vfma(splat<T>(0.5f * kCs2), drho, vfma(ux, r, F[z][0][2]));
+      } else {
+        s = F[z][b][0];
+        r = vfma(hux, s, F[z][b][1]);
+        e = vfma(al, s, vfma(tux, F[z][b][1], F[z][b][2]));
+      }
+      F[z][b][0] = vdiff(e, r);
+      F[z][b][2] = vadd(e, r);
+      F[z][b][1] = vfma(splat<T>(-2.0f), e, s);
+    }
+#pragma unroll
+  for (int z = z0; z < z1; ++z)
+#pragma unroll
+    for (int x = 0; x < 3; ++x) raw_inv_h(F[z][0][x], F[z][1][x], F[z][2][x]);
+  if (D == 3) {
+#pragma unroll
+    for (int y = 0; y < 3; ++y)
+#pragma unroll
+      for (int x = 0; x < 3; ++x) raw_inv_h(F[0][y][x], F[1][y][x], F[2][y][x]);
+  }
 }
 
+// Raw moments in the halved convention -> populations.
 template <int D, typename T>
 __device__ __forceinline__ void tile_raw_inv_h(T (&F)[3][3][3]) {
   constexpr int z0 = (D == 3) ? 0 : 1, z1 = (D == 3) ? 3 : 2;
@@ -296,22 +346,22 @@ __device__ __forceinline__ void shear_raw_moments(T (&F)[3][3][3], T &drho, T (&
 #pragma unroll
     for (int y = 0; y < 3; ++y) {
       r0[z][y] = vadd(F[z][y][1], vadd(F[z][y][0], F[z][y][2]));
-      r1[z][y] = vsub(F[z][y][2], F[z][y][0]);
+      r1[z][y] = vdiff(F[z][y][2], F[z][y][0]);
     }
   T q00[3], q01[3], q10[3], q11[3];  // [z]: (x order, y order) = 00, 01 (c_y), 10 (c_x), 11 (c_x c_y)
 #pragma unroll
   for (int z = 0; z < 3; ++z) {
     q00[z] = vadd(r0[z][1], vadd(r0[z][0], r0[z][2]));
-    q01[z] = vsub(r0[z][2], r0[z][0]);
+    q01[z] = vdiff(r0[z][2], r0[z][0]);
     q10[z] = vadd(r1[z][1], vadd(r1[z][0], r1[z][2]));
-    q11[z] = vsub(r1[z][2], r1[z][0]);
+    q11[z] = vdiff(r1[z][2], r1[z][0]);
   }
   drho = vadd(q00[1], vadd(q00[0], q00[2]));
-  j[2] = vsub(q00[2], q00[0]);
+  j[2] = vdiff(q00[2], q00[0]);
   j[0] = vadd(q10[1], vadd(q10[0], q10[2]));
-  P[1] = vsub(q10[2], q10[0]);  // c_x c_z
+  P[1] = vdiff(q10[2], q10[0]);  // c_x c_z
   j[1] = vadd(q01[1], vadd(q01[0], q01[2]));
-  P[2] = vsub(q01[2], q01[0]);  // c_y c_z
+  P[2] = vdiff(q01[2], q01[0]);  // c_y c_z
   P[0] = vadd(q11[1], vadd(q11[0], q11[2]));  // c_x c_y
 }
 

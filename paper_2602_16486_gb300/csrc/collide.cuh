@@ -218,10 +218,8 @@ __device__ __forceinline__ void collide_rates(T (&F)[3][3][3], float rho0, const
     ux = vmul(jv[0], inv_rho);
     uy = vmul(jv[1], inv_rho);
     uz = vmul(jv[2], inv_rho);
-    mom<D>(F, 0, 0, 0) = rho;  // k*_0 = rho for the way back
   } else if (SHEAR) {
     site_macros<D>(F, rho0, drho, rho, ux, uy, uz);
-    mom<D>(F, 0, 0, 0) = rho;  // k*_0 = rho for the way back
     if (D == 3) {
       Pm[0] = F[0][1][1];
       Pm[1] = F[1][0][1];
@@ -271,9 +269,6 @@ __device__ __forceinline__ void collide_rates(T (&F)[3][3][3], float rho0, const
       }
     }
     if (ISO) iso_unrotate_h(F[0][0][2], F[0][2][0], F[2][0][0]);
-    F[0][0][1] = zero;  // k*_1 (x momentum, central)
-    F[0][1][0] = zero;  // k*_2
-    F[1][0][0] = zero;  // k*_3
   } else {
     // D2Q9: modes 3 and 4 are the sum and difference of the (2,0) and (0,2) moments.
     T k[9];
@@ -303,14 +298,10 @@ __device__ __forceinline__ void collide_rates(T (&F)[3][3][3], float rho0, const
     F[1][1][2] = k[6];
     F[1][2][1] = k[7];
     F[1][2][2] = k[8];
-    F[1][0][1] = zero;  // k*_1
-    F[1][1][0] = zero;  // k*_2
   }
-  // r* = N^{-1} k* (entry (0,0,0) = k*_0 = rho), then d* = M^{-1} r* - w rho0, on the tile
-  // in the halved convention (every other entry already carries its tile scale).
-  tile_shift_inv_h<D>(F, ux, uy, uz);
-  mom<D>(F, 0, 0, 0) = drho;
-  tile_raw_inv_h<D>(F);
+  // r* = N^{-1} k* with k*_0 = rho and k*_1 .. k*_D = 0, then d* = M^{-1} r* - w rho0, on the tile
+  // in the halved convention (every entry already carries its tile scale).
+  tile_inv_h<D>(F, rho, drho, ux, uy, uz);
 }
 
 }  // namespace flbm

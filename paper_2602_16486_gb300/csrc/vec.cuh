@@ -6,6 +6,8 @@
 
 #include <cuda_runtime.h>
 
+#include <cstdint>
+
 namespace flbm {
 
 // Rounded on their own (never contracted), as the packed forms are: one site and two give the
@@ -26,6 +28,18 @@ __device__ __forceinline__ float2 vmul(float2 a, float2 b) { return __fmul2_rn(a
 __device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 vsub(float2 a, float2 b) {
   return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a);
+}
+
+// a - b where neither is a rounded product: the packed subtraction has one operand less to fetch than
+// the multiply-add of vsub, but the compiler contracts a product into it (D3Q27 64^3 9.63 -> 9.57 us a
+// step, 25x50x100 6.75 -> 6.65, D2Q9 4096^2 BF16 161.8 -> 160.7).
+__device__ __forceinline__ float vdiff(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float2 vdiff(float2 a, float2 b) {
+  const unsigned long long x = (unsigned long long)__float_as_uint(a.y) << 32 | __float_as_uint(a.x);
+  const unsigned long long y = (unsigned long long)__float_as_uint(b.y) << 32 | __float_as_uint(b.x);
+  unsigned long long r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(x), "l"(y));
+  return make_float2(__uint_as_float((uint32_t)r), __uint_as_float((uint32_t)(r >> 32)));
 }
 
 template <typename T>
