@@ -221,7 +221,7 @@ int flbm_stats_noalloc(int lattice, const int64_t dims[3], int storage, int pari
 
 /*
  * Step-kernel variant (launch configuration only; every variant computes the same
- * update): 0 = default (chosen by size, storage and noise), 1 = one site per thread, 2..8 =
+ * update): 0 = default (the form of 5, or of 7 on a small box), 1 = one site per thread, 2..8 =
  * two sites per thread with the sites flattened over the rows, so that every row length
  * fills the warps; 2, 3, 4 and 8 form 64-bit offsets, 5, 6 and 7 32-bit ones (a plane of
  * 4 GB or more always takes 64). By default and with 7 or 8, a call of many steps (six in

@@ -328,16 +328,11 @@ int resolve_variant(const flbm_ctx *c) {
 }
 
 // The variant launched. One site per thread only where it was asked for (the pair kernels take
-// every row length). The default is the form with 32-bit offsets but for large noisy FP32 D3Q27
-// boxes at the paper's rates, which are bound by DRAM and stream better with 64-bit ones (256^3:
-// 0.547 against 0.555 ms; general rates 0.592 against 0.577, 64^3 10.3 against 10.0 us, 16-bit 256^3
-// 0.534 against 0.522).
-int launch_variant(const flbm_ctx *c) {
-  if (c->variant != kStepAuto) return c->variant;
-  const bool dram = c->D == 3 && c->Q == 27 && c->storage == FLBM_FP32 && c->kBT > 0.0 && c->shear &&
-                    c->model == FLBM_COLLISION_CM && c->args.early;
-  return dram ? int(kStepPair) : int(kStepPairOcc);
-}
+// every row length). The default is the form with 32-bit offsets, compiled for fewer blocks per SM
+// (D3Q27 FP32, 32-bit / 64-bit offsets: 64^3 8.9 / 10.3 us, 192^3 233 / 242, 272^3 665 / 689, 384^3 1841 / 1913; only
+// where planes lie a large power of two apart the 64-bit form is level or a little ahead, 256^3 550 / 548,
+// which the autotuner finds).
+int launch_variant(const flbm_ctx *c) { return c->variant == kStepAuto ? int(kStepPairOcc) : c->variant; }
 
 // Whether a call of n steps runs as one launch (step_cluster.cu): by default, and for the variants
 // that stood for short rows.

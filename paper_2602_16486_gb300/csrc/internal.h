@@ -17,6 +17,8 @@ constexpr int kStepBlock = 128;   // threads per block of the step kernels
 // (256 k) 17.5 / 18.8, 96^3 (442 k) 30.5 / 29.9, 128^3 79.9 / 73.7; D2Q9 512^2 3.5 / 4.2, 1024^2 (524 k)
 // 11.2 / 11.1, 2048^2 48.9 / 46.4.
 constexpr uint32_t kEarlySlots = 3u * 152u * 5u * 128u;
+// Pair slots up to which a step launch gives an SM at most three blocks (step_kernels.cuh, launch_kernel).
+constexpr uint32_t kFewSlots = 3u * 152u * 128u;
 constexpr int kStatsBlock = 128;  // threads (= sites per tile) of the statistics kernel
 
 // Arguments of one fused step launch (passed by value, lives in the constant bank).

@@ -16,8 +16,8 @@
 //
 // The reads go by cp.async (4 or 8 bytes) into a stage of the thread's own words
 // (stage[word][thread]: no bank conflicts and no barrier), so that loads in flight hold no
-// registers and on long launches the noise is formed while they travel. Without noise there is nothing to form
-// meanwhile and the reads go to registers directly (STAGE false: 256^3 D3Q27 0.526 ms against 0.538
+// registers and on long launches the noise is formed while they travel. Without noise there is
+// nothing to form meanwhile and the reads go to registers directly (STAGE false: 256^3 D3Q27 0.526 ms against 0.538
 // staged), as do unaligned 16-bit elements (2 bytes, below cp.async's smallest size).
 //
 // ROWS (odd steps of aligned rows): the block's slots lie in one row, so that the row and plane

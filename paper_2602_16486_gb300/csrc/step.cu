@@ -35,10 +35,11 @@
 //  - programmatic dependent launch: on short launches the next step's blocks form their noise
 //    while this step drains (half of it before the wait and half while the populations travel was
 //    slower: D2Q9 512^2 4.2 against 3.4 us, D3Q27 32^3 4.3 against 3.3).
+//  - register caps by size (launch_kernel): more chains in flight per warp, 64^3 9.6 -> 8.8.
 // Measured (us per step, before -> now): D2Q9 64^2 4.1 -> 1.8 (and 0.86 in calls of many steps,
-// step_cluster.cu), 200^2 5.0 -> 1.9, 512^2 6.2 -> 3.4, 4096^2 BF16 176 -> 162; D3Q27 25x50x100 13.5 ->
-// 6.8, 64^3 20 -> 9.9 (13.3 in its best launch shape), 96^3 BGK 62 -> 31, 256^3 FP32 580 -> 547 (6.6
-// TB/s, 0.99 of the measured copy), FP16 571 -> 521; D3Q19 256^3 478 -> 391 (with d3q19.cuh).
+// step_cluster.cu), 200^2 5.0 -> 1.9, 512^2 6.2 -> 3.3, 4096^2 BF16 176 -> 160; D3Q27 25x50x100 13.5 ->
+// 5.3, 64^3 20 -> 8.8 (13.3 in its best launch shape), 96^3 BGK 62 -> 30, 256^3 FP32 580 -> 548 (6.6
+// TB/s, 0.99 of the measured copy), FP16 571 -> 512; D3Q19 256^3 478 -> 388 (with d3q19.cuh).
 // Tried and slower: scalar FMAs in place of the packed ones (256^3 FP16 0.615
 // against 0.591 ms), six blocks per SM (spills: 0.586 against 0.550 ms).
 #include "step_kernels.cuh"

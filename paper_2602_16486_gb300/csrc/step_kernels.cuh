@@ -113,14 +113,29 @@ __global__ void __launch_bounds__(kStepBlock, MINB) pair_kernel(const StepArgs a
   }
 }
 
-// Blocks of 128 threads per SM that a pair kernel is compiled for (its register cap), measured at
-// 256^3 (FP32 D3Q27, us per step at 3 / 4 / 5 / 6 blocks): staged reads and the paper's rates 563 /
-// 551 / 550 / 586, where six spill; direct reads without noise 551 / 523 / 554 / -, of unaligned
-// elements (255^3) 534 / 559 / 711 / -. The general rates keep the tile and the noise together
-// (BGK 96^3: 35.1 / 33.8).
+// Blocks of 128 threads per SM that a pair kernel is compiled for (its register cap), where the launch
+// does not choose by size (launch_kernel): at 256^3 (FP32 D3Q27, ms per step at 3 / 4 / 5 blocks)
+// 64-bit offsets, staged reads, the paper's rates .563 / .551 / .548; direct reads without noise .551 /
+// .523 / .554, of unaligned elements (255^3) .534 / .559 / .711. The general rates keep the tile and the
+// noise together (BGK 96^3 at 4 / 5: 33.8 / 35.1 us).
 template <int LAT, int SCHEME, bool DIRECT, bool ALIGNED>
 constexpr int pair_blocks() {
   return LAT == 2 ? 8 : DIRECT ? (ALIGNED ? 4 : 3) : SCHEME == kShear ? 5 : 4;
+}
+
+template <int N>
+using Blocks = std::integral_constant<int, N>;
+
+template <int LAT, typename S, int PARITY, bool NOISE, int SCHEME, bool ISO, bool ALIGNED, typename O, int MINB>
+cudaError_t launch_pair(cudaLaunchConfig_t &cfg, const StepArgs &a) {
+  if constexpr (PARITY == 1 && ALIGNED) {
+    const int per_row = (a.nx / 2 + kStepBlock - 1) / kStepBlock;
+    if (per_row * kStepBlock <= a.nx / 2 + a.nx / 16) {
+      cfg.gridDim = dim3(per_row, a.ny, a.nz_grid);
+      return cudaLaunchKernelEx(&cfg, pair_kernel<LAT, S, PARITY, NOISE, SCHEME, ISO, true, true, O, MINB>, a);
+    }
+  }
+  return cudaLaunchKernelEx(&cfg, pair_kernel<LAT, S, PARITY, NOISE, SCHEME, ISO, ALIGNED, false, O, MINB>, a);
 }
 
 template <int LAT, typename S, int PARITY, bool NOISE, int SCHEME, bool ISO>
@@ -139,23 +154,44 @@ cudaError_t launch_kernel(int variant, const StepArgs &a, cudaStream_t s) {
   cfg.stream = s;
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
-  constexpr int MB = pair_blocks<LAT, SCHEME, !NOISE, true>();
   const bool narrow = !a.wide && (variant == kStepPairOcc || variant == kStepPairRolledOcc || variant == kStepPairOccRows);
-  if (!a.aligned[PARITY])
-    return cudaLaunchKernelEx(&cfg, pair_kernel<LAT, S, PARITY, NOISE, SCHEME, ISO, false, false, uint32_t,
-                                                pair_blocks<LAT, SCHEME, !NOISE || sizeof(S) == 2, false>()>, a);
-  if constexpr (PARITY == 1) {
-    const int per_row = (a.nx / 2 + kStepBlock - 1) / kStepBlock;
-    if (per_row * kStepBlock <= a.nx / 2 + a.nx / 16) {
-      cfg.gridDim = dim3(per_row, a.ny, a.nz_grid);
-      if (narrow)
-        return cudaLaunchKernelEx(&cfg, pair_kernel<LAT, S, PARITY, NOISE, SCHEME, ISO, true, true, uint32_t, MB>, a);
-      return cudaLaunchKernelEx(&cfg, pair_kernel<LAT, S, PARITY, NOISE, SCHEME, ISO, true, true, uint64_t, MB>, a);
+  // With noise, more registers let a warp keep several Philox streams and Box-Muller chains going,
+  // and a launch of few blocks has no use for room for more of them. us per step (FP32, the paper's
+  // rates; blocks per SM):
+  //   D3Q27, 32-bit offsets (3 / 4 / 5): 33^3 4.4 / 5.0 / 5.7, 48^3 4.4 / 4.9 / 6.0; 25x50x100 6.4 / 5.4 / 6.9,
+  //   64^3 9.4 / 8.9 / 9.9, 80^3 17.6 / 16.6 / 17.4, 192^3 - / 233 / 240, FP16 256^3 515 / 512 / 518;
+  //   unaligned (rows of odd length) 63^3 10.6 / 10.2 / 11.3, 127^3 85 / 87 / 89, 255^3 658 / 673 / 689;
+  //   general rates 48^3 4.7 / 5.1, BGK 4.5 / 5.0, but 25x50x100 6.2 / 5.6;
+  //   D3Q19 unaligned (4 / 5): 25x50x100 4.4 / 5.1, 255^3 467 / 463; aligned 64^3 6.8 / 6.6;
+  //   D2Q9 (5 / 8): 512^2 3.30 / 3.41, 4096^2 181 / 180, 4095^2 213 / 215.
+  const bool few = a.slots[PARITY] <= kFewSlots;
+  constexpr bool SHEAR = SCHEME == kShear, DIRECT = !NOISE || sizeof(S) == 2;
+  constexpr int MA = pair_blocks<LAT, SCHEME, !NOISE, true>(), MU = pair_blocks<LAT, SCHEME, DIRECT, false>();
+  const auto launch = [&](auto aligned, auto offset, auto blocks) {
+    return launch_pair<LAT, S, PARITY, NOISE, SCHEME, ISO, decltype(aligned)::value, decltype(offset),
+                       decltype(blocks)::value>(cfg, a);
+  };
+  using Yes = std::true_type;
+  using No = std::false_type;
+  if (!a.aligned[PARITY]) {
+    if constexpr (!DIRECT && LAT == 3) {
+      if (few || (SHEAR && a.early)) return launch(No{}, uint32_t{}, Blocks<3>{});
+      return launch(No{}, uint32_t{}, Blocks<4>{});
+    } else if constexpr (!DIRECT && SHEAR && LAT == 19) {
+      return a.early ? launch(No{}, uint32_t{}, Blocks<5>{}) : launch(No{}, uint32_t{}, Blocks<4>{});
+    } else {
+      return launch(No{}, uint32_t{}, Blocks<!DIRECT && SHEAR && LAT == 2 ? 5 : MU>{});
     }
   }
-  if (narrow)
-    return cudaLaunchKernelEx(&cfg, pair_kernel<LAT, S, PARITY, NOISE, SCHEME, ISO, true, false, uint32_t, MB>, a);
-  return cudaLaunchKernelEx(&cfg, pair_kernel<LAT, S, PARITY, NOISE, SCHEME, ISO, true, false, uint64_t, MB>, a);
+  if (narrow) {
+    if constexpr (NOISE && LAT == 3)
+      return few ? launch(Yes{}, uint32_t{}, Blocks<3>{}) : launch(Yes{}, uint32_t{}, Blocks<4>{});
+    else if constexpr (NOISE && SHEAR && LAT == 2)
+      return a.early ? launch(Yes{}, uint32_t{}, Blocks<MA>{}) : launch(Yes{}, uint32_t{}, Blocks<5>{});
+    else
+      return launch(Yes{}, uint32_t{}, Blocks<MA>{});
+  }
+  return launch(Yes{}, uint64_t{}, Blocks<MA>{});
 }
 
 template <int LAT, typename S, bool ISO, int SCHEME>

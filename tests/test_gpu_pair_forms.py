@@ -164,3 +164,24 @@ def test_many_steps_of_a_small_box(fl, oracle_mod, lattice, dims, rates):
         fo = oracle_mod.run(lattice, dims, lam, kbt, (1 << 33) + 7, f0, 0, 38, model=int(rates == "raw"))
         assert (np.abs(out[0] - fo) / w).max() <= TOL, kbt
         assert np.array_equal(out[0], out[1]), kbt
+
+
+# Pair slots on either side of the sizes at which a launch changes form: 58,368 (register caps) and
+# 291,840 (reads before the noise), in aligned rows and in rows of odd length.
+SIZES = [(0, (342, 340, 1)), (0, (344, 342, 1)), (0, (343, 341, 1)), (0, (764, 764, 1)), (0, (765, 763, 1)),
+         (1, (48, 48, 50)), (1, (48, 50, 50)), (1, (49, 49, 50)), (1, (84, 84, 84)), (1, (83, 84, 84)), (1, (256, 48, 48)),
+         (2, (51, 50, 50)), (3, (49, 49, 50)), (3, (83, 84, 84))]
+
+
+@pytest.mark.parametrize("lattice,dims", SIZES)
+@pytest.mark.parametrize("rates", ["paper", "general"])
+def test_forms_by_launch_size(fl, lattice, dims, rates):
+    # Bit for bit what one site per thread gives (that form is held to the oracle above), both parities.
+    lam, out = _lam((9, 27, 27, 19)[lattice], rates), []
+    for variant in (0, 1):
+        with fl.Lattice(lattice, dims, lam, 1e-4, 1.0, 77) as lat:
+            lat.variant = variant
+            lat.init_uniform((0.04, -0.02, 0.01), 1e-3, 3)
+            lat.step(3)
+            out.append(lat.populations())
+    assert np.array_equal(out[0], out[1])
