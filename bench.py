@@ -79,7 +79,7 @@ def measured_peaks():
 
 # Sources the single-lattice step kernels are compiled from (a change to any of them
 # invalidates recorded DRAM counters).
-STEP_SOURCES = ("step.cu", "step_kernels.cuh", "step_pipe.cu", "async.cuh", "cm.cuh", "collide.cuh", "philox.cuh",
+STEP_SOURCES = ("step.cu", "step_kernels.cuh", "pair.cuh", "cm.cuh", "collide.cuh", "d3q19.cuh", "philox.cuh",
                 "lattice.cuh", "vec.cuh", "internal.h")
 
 
