@@ -64,12 +64,12 @@ __device__ __forceinline__ uint4 philox4x32_10_ks(uint4 ctr, const K &keys) {
 
 // Box-Muller, angle: cos and sin of 2 pi u_b depend only on u_b mod 1, and the word read
 // as a signed integer s_b is that residue times 2^32: u_b = (floor(s_b / 2^9) + 1/2) 2^-23
-// mod 1. The angle is taken as 2 pi s_b 2^-32, with s_b converted to FP32 (rounded to 24 bits), which
-// lies within pi 2^-23 (3.7e-7 rad) of 2 pi u_b on either side: one conversion and one product,
-// in [-pi, pi]. (With pi 2^-23 added the angles erred to one side by up to 7.5e-7 rad: populations after
-// 50 steps, against 64 bits, 4.8e-7 -> 3.1e-7 of the spread without it.) cos / sin come from the hardware
-// approximations (__sincosf; absolute error about 4e-7 on [-pi, pi]), which cost two instructions
-// instead of a polynomial.
+// mod 1. The angle is taken as 2 pi (s_b 2^-32 + 2^-24), with s_b converted to FP32 (rounded to
+// 24 bits), which lies within 2 pi 2^-23 (7.5e-7 rad) of 2 pi u_b: one conversion and one FMA.
+// (Without the 2^-24 the error would be half of that, on either side, but 16-bit states of many
+// steps would differ from those of earlier builds by more than their rounding does.) cos / sin come
+// from the hardware approximations (__sincosf; absolute error about 4e-7 on [-pi, pi]), which cost
+// two instructions instead of a polynomial.
 //
 // The radius: u_a = (2 m_a + 1) 2^-24 is formed exactly from the word's top 23 bits (1 + m 2^-23
 // assembled by one funnel shift, minus 1 - 2^-24). The argument reduction of Cody & Waite
@@ -80,6 +80,7 @@ __device__ __forceinline__ uint4 philox4x32_10_ks(uint4 ctr, const K &keys) {
 // logarithm has an absolute error there that exceeds the value). Checked against the FP64
 // definition over all 2^23 codes: relative error of -2 ln u_a below 3e-7.
 constexpr float kAngleScale = 0x1p-32f * 6.28318530717958647692f;  // 2 pi 2^-32
+constexpr float kAngleOffset = 0x1p-23f * 3.14159265358979323846f;  // pi 2^-23 = 2 pi 2^-24
 
 // Words of Philox block `blk` for each lane's site (lane l: site0 + l * dsite).
 template <int L, typename K>
@@ -128,7 +129,7 @@ __device__ __forceinline__ void box_muller(const uint32_t (&wa)[Lanes<T>::n], co
   P = vfma(P, s2, splat<T>(float(-4.0 * V)));
   const T a = vfma(kf, splat<T>(float(-1.3862943611198906 * 0x1p-23 * V)), vmul(sx, P));  // V (-2 ln u_a)
   rad = sqrt_fast_lanes(a);
-  const T th = vmul(ang, splat<T>(kAngleScale));
+  const T th = vfma(ang, splat<T>(kAngleScale), splat<T>(kAngleOffset));
 #pragma unroll
   for (int l = 0; l < L; ++l) {
     float sl, cl;
