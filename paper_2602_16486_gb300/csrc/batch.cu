@@ -66,7 +66,7 @@ __device__ __forceinline__ auto pair_of(const BatchLattice &L, const Base &plane
     p.init_flat(planes, 0u, L.plane, slot);
   } else {
     int x0, y, z;
-    slot_xyz(slot, L.nx, L.ny, L.m_hp, L.p_hp(), L.m_ny, L.p_ny(), x0, y, z);
+    slot_xyz<!ALIGNED && sizeof(O) == 8>(slot, L.nx, L.ny, L.m_hp, L.p_hp(), L.m_ny, L.p_ny(), x0, y, z);
     p.init_row(planes, x0, y, z, L.nx, L.ny, L.nz);
   }
   return p;

@@ -48,18 +48,25 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_prerequisites() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// Quotient x / d by the multiply-shift constants of batch_magic (internal.h), x < 2^31.
-__device__ __forceinline__ uint32_t udiv_magic(uint32_t x, uint32_t m, int p) {
-  return (uint32_t)(((unsigned long long)x * m) >> p);
+// Quotient x / d by the multiply-shift constants of batch_magic (internal.h): exact for x < 2^31, or
+// (ANY) for every x. ANY divides x / 2 and puts the last bit right, four more operations.
+template <bool ANY>
+__host__ __device__ __forceinline__ uint32_t udiv_magic(uint32_t x, uint32_t d, uint32_t m, int p) {
+  if (!ANY) return (uint32_t)(((unsigned long long)x * m) >> p);
+  const uint32_t q = 2u * (uint32_t)(((unsigned long long)(x >> 1) * m) >> p);
+  return x - q * d >= d ? q + 1u : q;
 }
 
-// Row coordinates of pair slot `slot` (rows of hp = ceil(nx / 2) slots).
-__device__ __forceinline__ void slot_xyz(uint32_t slot, int nx, int ny, uint32_t m_hp, int p_hp, uint32_t m_ny,
-                                         int p_ny, int &x0, int &y, int &z) {
+// Row coordinates of pair slot `slot` (rows of hp = ceil(nx / 2) slots). ANY: the slots may number 2^31
+// or more. That takes rows of odd length (nx = 1 has as many slots as sites, which are below 2^32) and
+// a plane of 4 GB or more, so the step kernels, which send such planes to one site per thread, do without.
+template <bool ANY>
+__host__ __device__ __forceinline__ void slot_xyz(uint32_t slot, int nx, int ny, uint32_t m_hp, int p_hp, uint32_t m_ny,
+                                                  int p_ny, int &x0, int &y, int &z) {
   const uint32_t hp = (uint32_t)((nx + 1) >> 1);
-  const uint32_t r = udiv_magic(slot, m_hp, p_hp);
+  const uint32_t r = udiv_magic<ANY>(slot, hp, m_hp, p_hp);
   x0 = 2 * (int)(slot - r * hp);
-  const uint32_t q = udiv_magic(r, m_ny, p_ny);
+  const uint32_t q = udiv_magic<ANY>(r, (uint32_t)ny, m_ny, p_ny);
   y = (int)(r - q * (uint32_t)ny);
   z = (int)q;
 }

@@ -63,7 +63,7 @@ __device__ __forceinline__ void load_pair(const StepArgs &a, uint32_t k, PairPop
       p.init_flat(PlaneTable{a.pop}, a.first, a.count, k);
     } else {
       int x0, y, z;
-      slot_xyz(k, a.nx, a.ny, a.m_hp, a.p_hp, a.m_ny, a.p_ny, x0, y, z);
+      slot_xyz<!ALIGNED>(k, a.nx, a.ny, a.m_hp, a.p_hp, a.m_ny, a.p_ny, x0, y, z);
       p.init_row(PlaneTable{a.pop}, x0, y, z + a.z_lo, a.nx, a.ny, a.nz);
     }
     if constexpr (LAT == 19)

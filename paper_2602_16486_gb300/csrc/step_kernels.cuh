@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(kStepBlock, MINB) pair_kernel(const StepArgs a
       p.init_flat(PlaneTable{a.pop}, a.first, a.count, slot);
     } else {
       int x0, y, z;
-      slot_xyz(slot, a.nx, a.ny, a.m_hp, a.p_hp, a.m_ny, a.p_ny, x0, y, z);
+      slot_xyz<false>(slot, a.nx, a.ny, a.m_hp, a.p_hp, a.m_ny, a.p_ny, x0, y, z);
       p.init_row(PlaneTable{a.pop}, x0, y, z + a.z_lo, a.nx, a.ny, a.nz);
     }
   }
