@@ -80,9 +80,9 @@ __device__ __forceinline__ void lattice_noise(float2 (&n)[Noisy<D>::count], cons
   const KeyBase keys{L.key0, L.key1};
   const uint32_t lo = (uint32_t)step, hi = (uint32_t)(step >> 32);
   if (SHEAR)
-    noise_modes<D, true, false, B0, B1>(n, ShearRates<D>{L.sqrt_kbt, L.om_shear, L.amp_shear}, s0, lo, hi, keys, dsite);
+    noise_modes<D, float, true, false, B0, B1>(n, ShearRates<D>{L.sqrt_kbt, L.om_shear, L.amp_shear}, s0, lo, hi, keys, dsite);
   else
-    noise_modes<D, false, false, B0, B1>(n, ArrayRates{rates, rates + 27, nullptr, 0.0f}, s0, lo, hi, keys, dsite);
+    noise_modes<D, float, false, false, B0, B1>(n, ArrayRates{rates, rates + 27, nullptr, 0.0f}, s0, lo, hi, keys, dsite);
 }
 template <int D, bool SHEAR>
 __device__ __forceinline__ void lattice_collide(float2 (&F)[3][3][3], const BatchLattice &L, const float *rates,

@@ -76,8 +76,8 @@ __host__ __device__ constexpr double csqrt(double x) {
   return r;
 }
 
-// n of the modes of Philox blocks [B0, B1).
-template <int LAT, bool SHEAR, bool ISO, int B0, int B1, typename T, typename R, typename K>
+// n of the modes of Philox blocks [B0, B1), for populations stored in S (philox.cuh, the angle).
+template <int LAT, typename S, bool SHEAR, bool ISO, int B0, int B1, typename T, typename R, typename K>
 __device__ __forceinline__ void noise_modes(T (&n)[Noisy<LAT>::count], const R &rates, uint32_t site0,
                                             uint32_t step_lo, uint32_t step_hi, const K &keys, uint32_t dsite) {
   constexpr int L = Lanes<T>::n, N = Noisy<LAT>::count, first = Noisy<LAT>::first;
@@ -97,7 +97,7 @@ __device__ __forceinline__ void noise_modes(T (&n)[Noisy<LAT>::count], const R &
       }
       const double V0 = SHEAR ? noise_variance<LAT, ISO>(first + m) : 1.0;
       T rad, c, s;
-      box_muller<T>(wa, wb, V0, rad, c, s);
+      box_muller<sizeof(S) == 2, T>(wa, wb, V0, rad, c, s);
       n[m] = vmul(rad, c);
       if constexpr (!SHEAR) n[m] = vmul(splat<T>(rates.phc(first + m)), n[m]);
       if (m + 1 < N) {

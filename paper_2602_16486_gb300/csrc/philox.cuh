@@ -64,12 +64,14 @@ __device__ __forceinline__ uint4 philox4x32_10_ks(uint4 ctr, const K &keys) {
 
 // Box-Muller, angle: cos and sin of 2 pi u_b depend only on u_b mod 1, and the word read
 // as a signed integer s_b is that residue times 2^32: u_b = (floor(s_b / 2^9) + 1/2) 2^-23
-// mod 1. The angle is taken as 2 pi (s_b 2^-32 + 2^-24), with s_b converted to FP32 (rounded to
-// 24 bits), which lies within 2 pi 2^-23 (7.5e-7 rad) of 2 pi u_b: one conversion and one FMA.
-// (Without the 2^-24 the error would be half of that, on either side, but 16-bit states of many
-// steps would differ from those of earlier builds by more than their rounding does.) cos / sin come
-// from the hardware approximations (__sincosf; absolute error about 4e-7 on [-pi, pi]), which cost
-// two instructions instead of a polynomial.
+// mod 1. The angle is 2 pi s_b 2^-32, with s_b converted to FP32 (rounded to 24 bits): s_b lies in
+// the interval of 2^9 words that has u_b in its middle, so this is within pi 2^-23 (3.7e-7 rad) of
+// 2 pi u_b on either side. Half an interval added to it (OFFSET, one FMA instead of the product) makes
+// that 0 to 2 pi 2^-23 and is most of the error of a noisy FP32 step: against 64 bits, with and without,
+// D3Q27 64^3 50 steps 4.9e-7 / 3.2e-7, D2Q9 512^2 5.0e-7 / 3.4e-7. States kept in 16 bits have errors of 2e-4
+// and more whatever the angle's last bits, which only move their roundings: there the offset stays.
+// cos / sin come from the hardware approximations (__sincosf; absolute error about 4e-7 on [-pi, pi]),
+// which cost two instructions instead of a polynomial.
 //
 // The radius: u_a = (2 m_a + 1) 2^-24 is formed exactly from the word's top 23 bits (1 + m 2^-23
 // assembled by one funnel shift, minus 1 - 2^-24). The argument reduction of Cody & Waite
@@ -97,7 +99,7 @@ __device__ __forceinline__ void philox_lanes(uint32_t site0, uint32_t step_lo, u
 // the minimax cubic on [0, 0.02944] (Remez exchange; relative error 7e-10, against the Taylor
 // quartic's 8e-8 s-dependent tail at one more multiply-add: the FP32 result is the same to its
 // rounding, 2.5e-7 over all 2^23 codes for both).
-template <typename T>
+template <bool OFFSET, typename T>
 __device__ __forceinline__ void box_muller(const uint32_t (&wa)[Lanes<T>::n], const uint32_t (&wb)[Lanes<T>::n],
                                            double V, T &rad, T &c, T &sn) {
   constexpr int L = Lanes<T>::n;
@@ -129,7 +131,7 @@ __device__ __forceinline__ void box_muller(const uint32_t (&wa)[Lanes<T>::n], co
   P = vfma(P, s2, splat<T>(float(-4.0 * V)));
   const T a = vfma(kf, splat<T>(float(-1.3862943611198906 * 0x1p-23 * V)), vmul(sx, P));  // V (-2 ln u_a)
   rad = sqrt_fast_lanes(a);
-  const T th = vfma(ang, splat<T>(kAngleScale), splat<T>(kAngleOffset));
+  const T th = OFFSET ? vfma(ang, splat<T>(kAngleScale), splat<T>(kAngleOffset)) : vmul(ang, splat<T>(kAngleScale));
 #pragma unroll
   for (int l = 0; l < L; ++l) {
     float sl, cl;

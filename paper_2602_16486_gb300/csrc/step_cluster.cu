@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(512) cluster_kernel(const StepArgs a, uint32_t
   float n[Noisy<LAT>::count];
   const auto noise = [&]() {
     if (NOISE && active)
-      site_noise<LAT, SCHEME, ISO, 0, Noisy<LAT>::blocks>(n, a, site, 0u, (uint32_t)step, (uint32_t)(step >> 32));
+      site_noise<LAT, float, SCHEME, ISO, 0, Noisy<LAT>::blocks>(n, a, site, 0u, (uint32_t)step, (uint32_t)(step >> 32));
   };
   cluster_arrive();
   noise();

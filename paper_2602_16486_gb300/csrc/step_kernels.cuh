@@ -23,10 +23,10 @@ template <int LAT>
 __device__ __forceinline__ ArrayRates rates_of(const StepArgs &a) {
   return LAT == 19 ? ArrayRates{a.om, a.phc, a.amp, a.sqrt_kbt} : ArrayRates{a.om_t, a.phc_t, a.amp, a.sqrt_kbt};
 }
-template <int LAT, int SCHEME, bool ISO, int B0, int B1, typename T>
+template <int LAT, typename S, int SCHEME, bool ISO, int B0, int B1, typename T>
 __device__ __forceinline__ void site_noise(T (&n)[Noisy<LAT>::count], const StepArgs &a, uint32_t site, uint32_t dsite,
                                            uint32_t step_lo, uint32_t step_hi) {
-  noise_modes<LAT, SCHEME == kShear, ISO, B0, B1>(n, rates_of<LAT>(a), site + a.site_base, step_lo, step_hi,
+  noise_modes<LAT, S, SCHEME == kShear, ISO, B0, B1>(n, rates_of<LAT>(a), site + a.site_base, step_lo, step_hi,
                                                   KeyTable{a.ks0, a.ks1}, dsite);
 }
 template <int LAT, bool NOISE, int SCHEME, bool ISO, typename T, typename F>
@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(kStepBlock) step_kernel(const StepArgs a) {
   S *__restrict__ f = static_cast<S *>(a.f);
   const uint32_t site = (uint32_t)(x + (long long)a.nx * (y + (long long)a.ny * z));
   float n[Noisy<LAT>::count];
-  if (NOISE) site_noise<LAT, SCHEME, ISO, 0, Noisy<LAT>::blocks>(n, a, site, 0u, a.step_lo, a.step_hi);
+  if (NOISE) site_noise<LAT, S, SCHEME, ISO, 0, Noisy<LAT>::blocks>(n, a, site, 0u, a.step_lo, a.step_hi);
   if constexpr (LAT == 19) {
     float F[19];
     load19<S, PARITY>(f, a.plane, nb, F);
@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(kStepBlock, MINB) pair_kernel(const StepArgs a
     wait_prerequisites();
     p.fetch(st);
   }
-  if (NOISE) site_noise<LAT, SCHEME, ISO, 0, B>(n, a, p.site0, p.dsite, a.step_lo, a.step_hi);
+  if (NOISE) site_noise<LAT, S, SCHEME, ISO, 0, B>(n, a, p.site0, p.dsite, a.step_lo, a.step_hi);
   if (!a.early) {
     wait_prerequisites();
     p.fetch(st);
