@@ -2,7 +2,7 @@
 // context and batch ownership, launch sequencing, graph capture of batch steps, the
 // autotuners and host <-> device exchange. Every compute step runs in the kernels of the
 // other translation units: the step (step.cu, step_16.cu, step_iso.cu, step19.cu,
-// step_pipe.cu), the statistics (stats.cu), initialisation and exchange (state.cu) and
+// step_raw.cu, step_cluster.cu), the statistics (stats.cu), initialisation and exchange (state.cu) and
 // batches (batch.cu).
 #include <cuda_runtime.h>
 
@@ -352,6 +352,8 @@ struct CkptHeader {
   uint64_t payload_bytes;
   int32_t model, pad;
 };
+// First field of the autotuner's keys: changes with the kernels that the variant numbers stand for.
+const char kTuneTag[] = "pairs1";
 const char kMagic[8] = {'F', 'L', 'B', 'M', 'C', 'K', 'P', '1'};
 
 }  // namespace
@@ -755,16 +757,20 @@ int flbm_autotune(flbm_ctx *c, int trial_steps, int *chosen) {
   if (c->slab) return fail(FLBM_ESTATE, "a slab is not tuned alone (its steps need halo exchanges)");
   if (trial_steps < 2) return fail(FLBM_EINVAL, "trial_steps must be >= 2");
   DeviceGuard g(c->device);
-  // Cache: one choice per (device, lattice, storage, nx parity, size class, noise, rate
-  // structure, collision model, rows shorter than one block).
+  // Cache: one choice per (device, lattice, storage, nx parity, size class, noise, rate structure,
+  // collision model, rows shorter than one block, one-launch form available). The tag names the set of
+  // kernels that the variant numbers stand for; lines of other sets match no key.
   cudaDeviceProp prop;
   FLBM_CUDA(cudaGetDeviceProperties(&prop, c->device));
+  // A small box's calls of many steps run in one launch: tried over enough of them to show it. The largest
+  // such box shares its size class with boxes that have no such form.
+  const bool small = cluster_applies(c->lattice, c->storage, c->N, 20);
   int size_class = 0;
   for (long long n = c->N; n > 1; n >>= 1) ++size_class;
   char key[320];
-  std::snprintf(key, sizeof(key), "%s|%d|%d|%d|%d|%d|%d|%d|%d", prop.name, c->lattice, c->storage,
+  std::snprintf(key, sizeof(key), "%s|%s|%d|%d|%d|%d|%d|%d|%d|%d|%d", kTuneTag, prop.name, c->lattice, c->storage,
                 int(c->dims[0] % 2), size_class, c->kBT > 0.0 ? 1 : 0, c->shear ? 1 : 0, c->model,
-                c->dims[0] < 2 * kStepBlock ? 1 : 0);
+                c->dims[0] < 2 * kStepBlock ? 1 : 0, small ? 1 : 0);
   static std::mutex mu;
   static std::map<std::string, int> cache;
   static bool file_read = false;
@@ -812,8 +818,6 @@ int flbm_autotune(flbm_ctx *c, int trial_steps, int *chosen) {
       st = fail(FLBM_ECUDA, "autotune set-up: %s", cudaGetErrorString(cudaGetLastError()));
       break;
     }
-    // A small box's calls of many steps run in one launch: tried over enough of them to show it.
-    const bool small = cluster_applies(c->lattice, c->storage, c->N, 20);
     if (small && trial_steps < 20) trial_steps = 20;
     for (int v : {int(kStepOneSite), int(kStepPair), int(kStepPairOcc), int(kStepPairOccRows)}) {
       if (v == kStepPairOccRows && !small) continue;
