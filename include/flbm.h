@@ -225,7 +225,8 @@ int flbm_stats_noalloc(int lattice, const int64_t dims[3], int storage, int pari
  * two sites per thread with the sites flattened over the rows, so that every row length
  * fills the warps; 2, 3, 4 and 8 form 64-bit offsets, 5, 6 and 7 32-bit ones (a plane of
  * 4 GB or more always takes 64). By default and with 7 or 8, a call of many steps (six in
- * 2-D, ten in 3-D) on a small FP32 box (8192 sites in 2-D, 4096 in 3-D) is one launch.
+ * 2-D, ten in 3-D) on a small FP32 box (8192 sites in 2-D, 4096 in 3-D) is one launch, where
+ * the device can place its up to 16 blocks as one cluster, and launches of 5 elsewhere.
  * flbm_get_step_variant reports 0 as 2, every choice as 1 when nx is odd (two sites per
  * thread run all the same, unless 1 was chosen), and 4 as 2 unless nx is even, at most 512
  * and a row of populations a multiple of 16 bytes.
@@ -244,6 +245,12 @@ int flbm_stats_noalloc(int lattice, const int64_t dims[3], int storage, int pari
  */
 int flbm_set_step_variant(flbm_ctx *ctx, int variant);
 int flbm_get_step_variant(const flbm_ctx *ctx);
+
+/*
+ * flbm_test_cluster_refused - test hook (the paper has no counterpart): with refused != 0 this
+ * context's steps run as on a device that cannot place the one-launch form.
+ */
+int flbm_test_cluster_refused(flbm_ctx *ctx, int refused);
 
 /*
  * Collision model of a context (default FLBM_COLLISION_CM, the paper's scheme).

@@ -51,6 +51,7 @@ struct flbm_ctx {
   long long *d_sites = nullptr;
   size_t sites_cap = 0;
   int variant = 0;  // enum StepVariant; 0 = default choice
+  bool test_no_cluster = false;  // flbm_test_cluster_refused
   bool shear = false;  // rates follow the paper's structure (collide.cuh, SHEAR)
   bool iso = false;    // the isotropic D3Q27 variant (lattice FLBM_D3Q27_ISO)
   StepArgs args{};
@@ -484,18 +485,23 @@ int flbm_step(flbm_ctx *c, int64_t n) {
                              "step taken from an odd step count, see flbm_slab_halo)");
   DeviceGuard g(c->device);
   const bool noise = c->kBT > 0.0;
-  if (takes_cluster(c, n)) {
-    for (int64_t left = n; left > 0;) {
-      const int k = int(left < (1 << 20) ? left : (1 << 20));
-      c->args.step_lo = uint32_t(uint64_t(c->step));
-      c->args.step_hi = uint32_t(uint64_t(c->step) >> 32);
-      FLBM_CUDA(launch_step_cluster(c->lattice, c->model == FLBM_COLLISION_RAW, noise, c->shear, c->args, k, c->stream));
+  int64_t left = n;
+  for (bool cluster = takes_cluster(c, n); cluster && left > 0;) {
+    const int k = int(left < (1 << 20) ? left : (1 << 20));
+    c->args.step_lo = uint32_t(uint64_t(c->step));
+    c->args.step_hi = uint32_t(uint64_t(c->step) >> 32);
+    const cudaError_t e = c->test_no_cluster ? cudaErrorNotSupported
+                                             : launch_step_cluster(c->lattice, c->model == FLBM_COLLISION_RAW, noise,
+                                                                   c->shear, c->args, k, c->stream);
+    if (e == cudaSuccess) {
       c->step += k;
       left -= k;
+    } else {
+      cudaGetLastError();  // launch by launch, then: an error that stays shows there
+      cluster = false;
     }
-    return FLBM_OK;
   }
-  for (int64_t s = 0; s < n; ++s) {
+  for (; left > 0; --left) {
     c->args.step_lo = uint32_t(uint64_t(c->step));
     c->args.step_hi = uint32_t(uint64_t(c->step) >> 32);
     if (c->model == FLBM_COLLISION_RAW)
@@ -733,6 +739,12 @@ int flbm_set_step_variant(flbm_ctx *c, int variant) {
   if (variant < kStepAuto || variant > kStepVariantMax)
     return fail(FLBM_EINVAL, "variant %d is not one of 0..%d", variant, int(kStepVariantMax));
   c->variant = variant;
+  return FLBM_OK;
+}
+
+int flbm_test_cluster_refused(flbm_ctx *c, int refused) {
+  if (!c) return fail(FLBM_EINVAL, "ctx is NULL");
+  c->test_no_cluster = refused != 0;
   return FLBM_OK;
 }
 

@@ -151,7 +151,8 @@ cudaError_t launch_step_d3q19(int storage, int variant, int parity, bool noise, 
 // The raw-moment collision (step_raw.cu): D 2 or 3.
 cudaError_t launch_step_raw(int D, int storage, int variant, int parity, bool noise, const StepArgs &a,
                             cudaStream_t s);
-// nsteps updates of a small FP32 box in one launch (step_cluster.cu), where cluster_applies.
+// nsteps updates of a small FP32 box in one launch (step_cluster.cu), where cluster_applies; an error
+// (nothing launched) where the device cannot place the cluster.
 bool cluster_applies(int lattice, int storage, long long sites, long long nsteps);
 cudaError_t launch_step_cluster(int lattice, bool raw, bool noise, bool shear, const StepArgs &a, int nsteps,
                                 cudaStream_t s);

@@ -20,6 +20,7 @@
 // Only 16 SMs work, so the rule (cluster_applies) ends where the whole GPU is faster.
 #include <map>
 #include <mutex>
+#include <utility>
 
 #include "step_kernels.cuh"
 
@@ -145,18 +146,23 @@ cudaError_t launch(const StepArgs &a, int nsteps, cudaStream_t s) {
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
   {
-    // More than eight blocks need the kernel's permission, once per device.
+    // More than eight blocks need the kernel's permission, and a device (or a partition of one) may
+    // have no group of SMs that holds them all: asked once per device and number of blocks.
     static std::mutex mu;
-    static std::map<int, bool> ready;
+    static std::map<std::pair<int, int>, bool> fits;
     int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    const cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     std::lock_guard<std::mutex> lock(mu);
-    if (!ready[dev]) {
-      e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-      if (e != cudaSuccess) return e;
-      ready[dev] = true;
+    const auto known = fits.find({dev, blocks});
+    bool ok = known != fits.end() && known->second;
+    if (known == fits.end()) {
+      int clusters = 0;
+      ok = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+           cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) == cudaSuccess && clusters > 0;
+      fits[{dev, blocks}] = ok;
     }
+    if (!ok) return cudaErrorNotSupported;
   }
   return cudaLaunchKernelEx(&cfg, kernel, a, chunk, nsteps);
 }

@@ -115,6 +115,7 @@ def _load():
         "flbm_sync": (ctypes.c_int, [vp]),
         "flbm_set_step_variant": (ctypes.c_int, [vp, ctypes.c_int]),
         "flbm_get_step_variant": (ctypes.c_int, [vp]),
+        "flbm_test_cluster_refused": (ctypes.c_int, [vp, ctypes.c_int]),
         "flbm_set_collision": (ctypes.c_int, [vp, ctypes.c_int]),
         "flbm_get_collision": (ctypes.c_int, [vp]),
         "flbm_autotune": (ctypes.c_int, [vp, ctypes.c_int, ctypes.POINTER(ctypes.c_int)]),
@@ -346,6 +347,10 @@ def flbm_stats_noalloc(lattice, dims, storage, parity, rho0, dev_populations, cu
 
 def flbm_set_step_variant(ctx, variant):
     _check(_lib.flbm_set_step_variant(ctx, int(variant)))
+
+
+def flbm_test_cluster_refused(ctx, refused):
+    _check(_lib.flbm_test_cluster_refused(ctx, int(refused)))
 
 
 def flbm_get_step_variant(ctx):
