@@ -226,10 +226,10 @@ int flbm_stats_noalloc(int lattice, const int64_t dims[3], int storage, int pari
  * fills the warps; 2, 3, 4 and 8 form 64-bit offsets, 5, 6 and 7 32-bit ones (a plane of
  * 4 GB or more always takes 64). By default and with 7 or 8, a call of many steps (six in
  * 2-D, ten in 3-D) on a small FP32 box (8192 sites in 2-D, 4096 in 3-D) is one launch, where
- * the device can place its up to 16 blocks as one cluster, and launches of 5 elsewhere.
- * flbm_get_step_variant reports 0 as 2, every choice as 1 when nx is odd (two sites per
- * thread run all the same, unless 1 was chosen), and 4 as 2 unless nx is even, at most 512
- * and a row of populations a multiple of 16 bytes.
+ * the device can place its up to 16 blocks as one cluster, and single launches elsewhere.
+ * flbm_get_step_variant reports the choice, and 0 as the form it is (5, or 7 on a small
+ * box), so that setting what it reports changes nothing (4 on a slab is reported as 2,
+ * whose launches it takes).
  * The environment variable FLBM_STEP_VARIANT, read by flbm_create, sets the initial
  * choice.
  * flbm_autotune times variants 1, 2 and 5 (and 7 on such a box, each over 20 steps at
@@ -261,8 +261,8 @@ int flbm_test_cluster_refused(flbm_ctx *ctx, int refused);
  * every non-conserved rate equal to omega it is the fluctuating BGK step of Sec. II-A:
  * f* = f + omega (f^eq - f) + zeta with zeta_i = w_i sum_v b_v^-1 M_vi phi_v eta_v
  * (Eq. Xi_pop). Available for FLBM_D2Q9 and FLBM_D3Q27 (FLBM_EINVAL otherwise), not for the
- * lattices of a batch (FLBM_ESTATE); flbm_get_step_variant reports every variant but 1 as 2. Statistics still report the central moments of the orthogonal basis. The model is
- * saved in checkpoints. Takes effect at the next flbm_step.
+ * lattices of a batch (FLBM_ESTATE). Statistics still report the central moments of the
+ * orthogonal basis. The model is saved in checkpoints. Takes effect at the next flbm_step.
  */
 enum flbm_collision { FLBM_COLLISION_CM = 0, FLBM_COLLISION_RAW = 1 };
 int flbm_set_collision(flbm_ctx *ctx, int model);

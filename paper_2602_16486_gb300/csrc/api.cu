@@ -109,9 +109,6 @@ int d_of(int lattice) { return lattice == FLBM_D2Q9 ? 2 : 3; }
 // Lattice code of the state, exchange and statistics kernels: 2 (D2Q9), 3 (D3Q27, both
 // bases) or 19 (D3Q19).
 int klat(int lattice) { return lattice == FLBM_D2Q9 ? 2 : (lattice == FLBM_D3Q19 ? 19 : 3); }
-// Lattices whose step kernels exist for variants 1, 2 and 5 only.
-bool pair_variants_only(int lattice) { return lattice == FLBM_D3Q27_ISO || lattice == FLBM_D3Q19; }
-
 int check_geometry(int lattice, const int64_t dims[3], int storage) {
   if (lattice != FLBM_D2Q9 && lattice != FLBM_D3Q27 && lattice != FLBM_D3Q27_ISO && lattice != FLBM_D3Q19)
     return fail(FLBM_EINVAL,
@@ -304,30 +301,6 @@ int enqueue_stats(flbm_ctx *c, double *record) {
   return FLBM_OK;
 }
 
-// Whether variant 4 takes the box (even rows of at most 512 sites, of whole 16-byte words,
-// two stages of which fit in shared memory); otherwise the choice counts as 2.
-bool long_rows_fit(const flbm_ctx *c) {
-  const size_t row = size_t(c->dims[0]) * storage_bytes(c->storage);
-  return c->dims[0] % 2 == 0 && c->dims[0] <= 512 && row % 16 == 0 &&
-         2 * size_t(c->D == 3 ? 27 : 9) * row + 16 <= 232448;
-}
-
-// The variant as flbm_get_step_variant reports it: the choice, or the default (two sites per
-// thread where nx is even, else one).
-int resolve_variant(const flbm_ctx *c) {
-  if (c->model == FLBM_COLLISION_RAW)  // raw-moment kernels: one site or two per thread
-    return c->dims[0] % 2 != 0 || c->variant == kStepOneSite ? int(kStepOneSite) : int(kStepPair);
-  int v = c->variant;
-  if (v == kStepAuto) v = kStepPair;
-  if (v == kStepPipelined && (!long_rows_fit(c) || c->slab)) v = kStepPair;
-  if (pair_variants_only(c->lattice)) {
-    if (v == kStepPairRolled || v == kStepPipelined) v = kStepPair;
-    if (v == kStepPairRolledOcc) v = kStepPairOcc;
-  }
-  if (v != kStepOneSite && c->dims[0] % 2 != 0) v = kStepOneSite;
-  return v;
-}
-
 // The variant launched. One site per thread only where it was asked for (the pair kernels take
 // every row length). The default is the form with 32-bit offsets, compiled for fewer blocks per SM
 // (D3Q27 FP32, 32-bit / 64-bit offsets: 64^3 8.9 / 10.3 us, 192^3 233 / 242, 272^3 665 / 689, 384^3 1841 / 1913; only
@@ -340,6 +313,14 @@ int launch_variant(const flbm_ctx *c) { return c->variant == kStepAuto ? int(kSt
 bool takes_cluster(const flbm_ctx *c, int64_t n) {
   return (c->variant == kStepAuto || c->variant == kStepPairOccRows || c->variant == kStepPairRows) && !c->slab &&
          cluster_applies(c->lattice, c->storage, c->N, n);
+}
+
+// The variant as flbm_get_step_variant reports it, such that setting it again changes nothing: the
+// choice, or for the default the variant it is. (4 on a slab is reported as 2, which it runs as.)
+int resolve_variant(const flbm_ctx *c) {
+  if (c->variant == kStepAuto)
+    return !c->slab && cluster_applies(c->lattice, c->storage, c->N, INT64_MAX) ? int(kStepPairOccRows) : int(kStepPairOcc);
+  return c->variant == kStepPipelined && c->slab ? int(kStepPair) : c->variant;
 }
 
 struct CkptHeader {
