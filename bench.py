@@ -439,7 +439,7 @@ def noise_off(fl, torch, stream, dims, peak, noisy_ms):
 
 
 FORMS = ["per-step launches", "persistent launch", "per-step launches, 5 blocks/SM (D2Q9: 10)",
-         "per-step launches, rolled noise loop"]
+         "per-step launches"]
 
 
 def batched_ensemble(fl, torch, peak, steps=200, calls=25):
@@ -685,7 +685,7 @@ def main(argv=None):
                    help="box for profiling runs (default 256,256,256: the workload)")
     p.add_argument("--no-e2e", action="store_true", help="skip the end-to-end leg (profiling runs)")
     p.add_argument("--variant", type=int, default=0,
-                   help="step-kernel variant (1-6); default 0 = autotune")
+                   help="step-kernel variant (1-8); default 0 = autotune")
     p.add_argument("--no-extras", action="store_true",
                    help="skip the 16-bit storage, other-lattice and batched-ensemble measurements")
     p.add_argument("--noise-off", action="store_true",

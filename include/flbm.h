@@ -356,19 +356,19 @@ int64_t flbm_batch_get_step(const flbm_batch *b);
 /*
  * Launch shape: threads per block (64, 128 or 256; every block takes tiles of
  * 2 * threads sites; 0 = the default, 128) and the form:
- *   0 per-step launches, up to 128 registers, D3Q27 noise loop unrolled (default);
- *   1 persistent cooperative launch (rolled noise loop, both lattice types in one kernel);
+ *   0 per-step launches, up to 128 registers (D2Q9: 64; the default);
+ *   1 persistent cooperative launch (both lattice types in one kernel);
  *   2 per-step launches compiled for more resident blocks per SM: five for D3Q27 (up
  *     to 102 registers), ten for D2Q9 (up to 51); threads <= 128;
- *   3 per-step launches, up to 128 registers, D3Q27 noise loop rolled (smaller code).
+ *   3 the launches of 0.
  * flbm_batch_set_shape sets the shape of every lattice type; flbm_batch_get_shape
  * returns the D3Q27 lattices' one. In the per-step forms each lattice type (FLBM_D2Q9,
  * FLBM_D3Q27) launches separately and may take its own threads and per-step form
  * (flbm_batch_set_type_shape: form 0, 2 or 3; FLBM_ESTATE while the batch is in the
  * persistent form, which launches every type alike); flbm_batch_get_type_shape returns a
  * type's shape as launched.
- * flbm_batch_autotune times every (form, threads) pair for all lattices alike and then,
- * in a per-step form, every per-step shape of the D2Q9 lattices with the D3Q27 lattices'
+ * flbm_batch_autotune times every (form, threads) pair (but form 3) for all lattices alike and
+ * then, in a per-step form, every per-step shape of the D2Q9 lattices with the D3Q27 lattices'
  * shape fixed, over trial_steps steps each (rounded up to even) on a copy of the state
  * (restored afterwards, step count unchanged); keeps the fastest and returns the D3Q27
  * lattices' shape in *threads and *form (either may be NULL). Needs one extra copy of all

@@ -1372,7 +1372,7 @@ int flbm_batch_autotune(flbm_batch *b, int trial_steps, int *threads_out, int *f
     // Every lattice alike, then, in a per-step form, the D2Q9 lattices' own shape.
     for (int f = 0; f <= kBatchFormMax && st == FLBM_OK; ++f) {
       for (int t : {64, 128, 256}) {
-        if (f == kBatchStepOcc && t > 128) continue;
+        if (f == kBatchStepAlias || (f == kBatchStepOcc && t > 128)) continue;
         float ms = 0.0f;
         if ((st = trial(t, f, t, f, &ms)) != FLBM_OK) break;
         if (ms < best) {
@@ -1384,7 +1384,7 @@ int flbm_batch_autotune(flbm_batch *b, int trial_steps, int *threads_out, int *f
     }
     if (st == FLBM_OK && best_f != kBatchPersistent && b->g2.ntiles > 0 && b->g3.ntiles > 0) {
       const int t3 = best_t, f3 = best_f;
-      for (int f : {int(kBatchStep), int(kBatchStepOcc), int(kBatchStepRolled)}) {
+      for (int f : {int(kBatchStep), int(kBatchStepOcc)}) {
         for (int t : {64, 128, 256}) {
           if ((f == kBatchStepOcc && t > 128) || (t == t3 && f == f3)) continue;
           float ms = 0.0f;

@@ -108,10 +108,10 @@ struct BatchGroup {
 };
 // Launch forms of a batch (values of flbm_batch_set_shape's `form`).
 enum BatchForm {
-  kBatchStep = 0,        // per-step launches, 128-register cap, unrolled D3Q27 noise
+  kBatchStep = 0,        // per-step launches, 128-register cap (D2Q9: 64)
   kBatchPersistent = 1,  // one cooperative launch, per-lattice completion counters
   kBatchStepOcc = 2,     // per-step launches, five (D3Q27) / ten (D2Q9) blocks of <= 128 per SM
-  kBatchStepRolled = 3,  // per-step launches, 128-register cap, rolled D3Q27 noise
+  kBatchStepAlias = 3,   // launches of kBatchStep (accepted, never tried by the autotuner)
   kBatchFormMax = 3
 };
 // n steps as plain launches (per step one launch per lattice type, block = tile, each
