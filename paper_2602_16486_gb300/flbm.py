@@ -50,18 +50,30 @@ class flbm_stats_t(ctypes.Structure):
         return _record_dict(np.frombuffer(self, dtype=np.float64))
 
 
-# The struct as doubles: three 64-bit and two 32-bit integers, then the floating-point fields.
+# The struct as words of 8 bytes (the integers among them 64-bit, or 32-bit in words of 4).
 _RECORD_DOUBLES = ctypes.sizeof(flbm_stats_t) // 8
+
+
+def _words(field, size=8):
+    f = getattr(flbm_stats_t, field)
+    return f.offset // size, (f.offset + f.size) // size
+
+
+(_STEP, _), (_SITES, _), (_NONFINITE, _), (_MASS, _) = (_words(f) for f in ("step", "sites", "nonfinite", "mass"))
+(_LATTICE, _), (_Q, _) = _words("lattice", 4), _words("q", 4)
+_MOM, _U_MEAN, _UU = (slice(*_words(f)) for f in ("mom", "u_mean", "uu"))
+(_K_MEAN, _), (_K_COV, _) = _words("k_mean"), _words("k_cov")
 
 
 def _record_dict(a):
     """One record (a row of _RECORD_DOUBLES doubles) as a dict; the arrays are copies."""
-    step, sites, nonfinite = a[:3].view(np.int64).tolist()
-    lattice, q = a[3:4].view(np.int32).tolist()
+    i64, i32 = a.view(np.int64), a.view(np.int32)
+    q = int(i32[_Q])
     return {
-        "step": step, "sites": sites, "nonfinite": nonfinite, "lattice": lattice, "q": q, "mass": float(a[4]),
-        "mom": a[5:8].copy(), "u_mean": a[8:11].copy(), "uu": a[11:17].copy(), "k_mean": a[17:17 + q].copy(),
-        "k_cov": a[44:44 + q * q].reshape(q, q).copy(),
+        "step": int(i64[_STEP]), "sites": int(i64[_SITES]), "nonfinite": int(i64[_NONFINITE]),
+        "lattice": int(i32[_LATTICE]), "q": q, "mass": float(a[_MASS]),
+        "mom": a[_MOM].copy(), "u_mean": a[_U_MEAN].copy(), "uu": a[_UU].copy(),
+        "k_mean": a[_K_MEAN:_K_MEAN + q].copy(), "k_cov": a[_K_COV:_K_COV + q * q].reshape(q, q).copy(),
     }
 
 
