@@ -76,11 +76,10 @@ __device__ __forceinline__ uint4 philox4x32_10_ks(uint4 ctr, const K &keys) {
 // The radius: u_a = (2 m_a + 1) 2^-24 is formed exactly from the word's top 23 bits (1 + m 2^-23
 // assembled by one funnel shift, minus 1 - 2^-24). The argument reduction of Cody & Waite
 // (Software Manual for the Elementary Functions, 1980) writes u_a = 2^k x with x in
-// [sqrt(1/2), sqrt(2)), and ln x = 2 atanh(s) = 2 (s + s^3/3 + ... + s^9/9),
-// s = (x - 1)/(x + 1), |s| < 0.172 (truncation below 1e-9 relative). x - 1 is exact,
-// so the result keeps its relative accuracy as u_a -> 1, where r -> 0 (a hardware
-// logarithm has an absolute error there that exceeds the value). Checked against the FP64
-// definition over all 2^23 codes: relative error of -2 ln u_a below 3e-7.
+// [sqrt(1/2), sqrt(2)), and ln x = 2 atanh(s), s = (x - 1)/(x + 1), |s| < 0.172, a cubic in s^2
+// times s (box_muller). x - 1 is exact, so the result keeps its relative accuracy as u_a -> 1, where
+// r -> 0 (a hardware logarithm has an absolute error there that exceeds the value). Checked against
+// the FP64 definition over all 2^23 codes: relative error of -2 ln u_a below 3e-7.
 constexpr float kAngleScale = 0x1p-32f * 6.28318530717958647692f;  // 2 pi 2^-32
 constexpr float kAngleOffset = 0x1p-23f * 3.14159265358979323846f;  // pi 2^-23 = 2 pi 2^-24
 
@@ -96,9 +95,10 @@ __device__ __forceinline__ void philox_lanes(uint32_t site0, uint32_t step_lo, u
 // The Box-Muller pair of words (wa, wb): radius r = sqrt(V (-2 ln u_a)) and the cosine and
 // sine of the angle. V (a variance, compile-time when it is a literal) costs nothing: it
 // scales the constants of the logarithm. The series of -2 ln x / s = -4 atanh(s) / s in s^2 is
-// the minimax cubic on [0, 0.02944] (Remez exchange; relative error 7e-10, against the Taylor
-// quartic's 8e-8 s-dependent tail at one more multiply-add: the FP32 result is the same to its
-// rounding, 2.5e-7 over all 2^23 codes for both).
+// a minimax cubic on [0, 0.02944] (Remez exchange, the constant term fixed): relative error 1.4e-9,
+// 1.6e-9 with the coefficients rounded to FP32, against 2.0e-9 of the Taylor quartic at one more
+// multiply-add. Both are far below FP32 rounding, and the result is within 2.5e-7 of -2 ln u_a over
+// all 2^23 codes with either.
 template <bool OFFSET, typename T>
 __device__ __forceinline__ void box_muller(const uint32_t (&wa)[Lanes<T>::n], const uint32_t (&wb)[Lanes<T>::n],
                                            double V, T &rad, T &c, T &sn) {
