@@ -175,9 +175,9 @@ cudaError_t launch_noise(bool noise, const StepArgs &a, int nsteps, cudaStream_t
 }  // namespace
 
 // Up to 512 threads a block in 2-D, 256 in 3-D (27 populations of 256 sites: 27 KB of shared memory).
-// us per step over 100 steps, cluster against pair kernel: D2Q9 64^2 0.86 / 1.84, 90^2 1.26 / 1.88; D3Q27 8^3 1.35 / 2.75, 16^3 1.99 / 2.92, 18^3 2.92 / 3.03; D3Q19
-// 16^3 1.49 / 2.40. Setting up the cluster takes some 10 us: over 6 steps D2Q9 90^2 2.7 / 2.8, D3Q27 16^3
-// 3.9 / 3.8, over 10 steps 2.1 / 2.5 and 3.0 / 3.5.
+// us per step over 100 steps, cluster against pair kernel: D2Q9 64^2 0.86 / 1.84, 90^2 1.26 / 1.88; D3Q27
+// 8^3 1.35 / 2.75, 16^3 1.99 / 2.92, 18^3 2.92 / 3.03; D3Q19 16^3 1.49 / 2.40. Setting up the cluster takes
+// some 10 us: over 6 steps D2Q9 90^2 2.7 / 2.8, D3Q27 16^3 3.9 / 3.8, over 10 steps 2.1 / 2.5 and 3.0 / 3.5.
 bool cluster_applies(int lattice, int storage, long long sites, long long nsteps) {
   return storage == 0 && sites <= (lattice == 0 ? 8192 : 4096) && nsteps >= (lattice == 0 ? 6 : 10);
 }
