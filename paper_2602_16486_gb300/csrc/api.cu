@@ -166,7 +166,7 @@ void fill_args(flbm_ctx *c) {
   a.aligned[0] = c->N % 2 == 0 && a.first % 2 == 0 && a.count % 2 == 0;
   a.aligned[1] = row % 2 == 0;
   a.wide = uint64_t(c->N) * storage_bytes(c->storage) > 0xFFFFFFFFull;
-  batch_magic(uint32_t((a.nx + 1) / 2), &a.m_hp, &a.p_hp);
+  batch_magic((uint32_t(a.nx) + 1) / 2, &a.m_hp, &a.p_hp);
   batch_magic(uint32_t(a.ny), &a.m_ny, &a.p_ny);
   a.early = a.slots[0] > kEarlySlots;
   a.sqrt_kbt = float(std::sqrt(c->kBT));
@@ -950,7 +950,7 @@ int batch_params(flbm_batch *b) {
     L.nz = a.nz;
     uint32_t m = 0;
     int p_hp = 0, p_ny = 0;
-    batch_magic(uint32_t((a.nx + 1) / 2), &L.m_hp, &p_hp);
+    batch_magic((uint32_t(a.nx) + 1) / 2, &L.m_hp, &p_hp);
     batch_magic(uint32_t(a.ny), &m, &p_ny);
     L.m_ny = m;
     L.dpp = uint32_t(c->D) | (uint32_t(p_hp) << 8) | (uint32_t(p_ny) << 16);

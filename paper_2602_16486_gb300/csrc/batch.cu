@@ -51,7 +51,7 @@ namespace {
 // tile spans rows and a warp's accesses stay contiguous for every nx. From an even step count
 // slot k is the flat sites 2k and 2k + 1 instead, and the last slots of odd rows stay empty.
 __device__ __forceinline__ uint32_t pair_slots(const BatchLattice &L) {
-  return (uint32_t)((L.nx + 1) >> 1) * (uint32_t)L.ny * (uint32_t)L.nz;
+  return (((uint32_t)L.nx + 1u) >> 1) * (uint32_t)L.ny * (uint32_t)L.nz;
 }
 template <int PARITY>
 __device__ __forceinline__ bool pairs_aligned(const BatchLattice &L) {

@@ -63,12 +63,19 @@ __host__ __device__ __forceinline__ uint32_t udiv_magic(uint32_t x, uint32_t d, 
 template <bool ANY>
 __host__ __device__ __forceinline__ void slot_xyz(uint32_t slot, int nx, int ny, uint32_t m_hp, int p_hp, uint32_t m_ny,
                                                   int p_ny, int &x0, int &y, int &z) {
-  const uint32_t hp = (uint32_t)((nx + 1) >> 1);
+  const uint32_t hp = ((uint32_t)nx + 1u) >> 1;
   const uint32_t r = udiv_magic<ANY>(slot, hp, m_hp, p_hp);
   x0 = 2 * (int)(slot - r * hp);
   const uint32_t q = udiv_magic<ANY>(r, (uint32_t)ny, m_ny, p_ny);
   y = (int)(r - q * (uint32_t)ny);
   z = (int)q;
+}
+
+// First site of pair slot k of a row; false past the row's end. A row has up to 2^31 - 1 sites and a launch
+// up to a block of slots more, whose sites are not ints any more.
+__host__ __device__ __forceinline__ bool row_slot(uint32_t k, int nx, int &x0) {
+  x0 = (int)(2u * k);
+  return 2u * k < (uint32_t)nx;
 }
 
 template <int LAT>

@@ -69,8 +69,8 @@ __global__ void __launch_bounds__(kStepBlock, MINB) pair_kernel(const StepArgs a
   launch_dependents();
   Access p;
   if (ROWS) {
-    const int x0 = 2 * (int)(blockIdx.x * kStepBlock + threadIdx.x);
-    if (x0 >= a.nx) return;
+    int x0;
+    if (!row_slot(blockIdx.x * (uint32_t)kStepBlock + threadIdx.x, a.nx, x0)) return;
     p.init_row(PlaneTable{a.pop}, x0, blockIdx.y, blockIdx.z + a.z_lo, a.nx, a.ny, a.nz);
   } else {
     const uint32_t slot = blockIdx.x * (uint32_t)kStepBlock + threadIdx.x;

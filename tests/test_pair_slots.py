@@ -18,14 +18,19 @@ DRIVER = r"""
 #include <cstdio>
 #include "internal.h"
 #include "pair.cuh"
-// Reads lines "nx ny slot any" and prints "x0 y z".
+// Reads lines "nx ny slot any" and prints "x0 y z"; any = 2: a slot of a row, "x0 in-the-row 0".
 int main() {
   int nx, ny, any;
   unsigned slot;
   while (std::scanf("%d %d %u %d", &nx, &ny, &slot, &any) == 4) {
     uint32_t m_hp, m_ny;
     int p_hp, p_ny, x0, y, z;
-    flbm::batch_magic(uint32_t((nx + 1) / 2), &m_hp, &p_hp);
+    if (any == 2) {
+      const bool in = flbm::row_slot(slot, nx, x0);
+      std::printf("%d %d 0\n", in ? x0 : 0, int(in));
+      continue;
+    }
+    flbm::batch_magic((uint32_t(nx) + 1) / 2, &m_hp, &p_hp);
     flbm::batch_magic(uint32_t(ny), &m_ny, &p_ny);
     if (any)
       flbm::slot_xyz<true>(slot, nx, ny, m_hp, p_hp, m_ny, p_ny, x0, y, z);
@@ -41,7 +46,8 @@ int main() {
 def _cases():
     rng = random.Random(3)
     boxes = [(1, 65534, 32773), (1, 65535, 65535), (1, 65533, 65535), (1, 40000, 65535), (3, 65535, 21845),
-             (5, 60001, 14000), (4001, 1021, 1051), (2, 65535, 32767), (65535, 65535, 1), (7, 5, 3), (1, 1, 1)]
+             (5, 60001, 14000), (4001, 1021, 1051), (2, 65535, 32767), (65535, 65535, 1), (7, 5, 3), (1, 1, 1),
+             (2 ** 31 - 1, 1, 1), (2 ** 31 - 2, 2, 1)]
     for _ in range(60):
         nx, ny = 2 * rng.randrange(40) + 1, rng.randrange(1, 65536)
         boxes.append((nx, ny, max(1, min(65535, (2 ** 32 - 1) // (nx * ny)))))
@@ -57,6 +63,10 @@ def _cases():
             yield nx, ny, s, 1, want
             if s < 2 ** 31:
                 yield nx, ny, s, 0, want
+    # A launch over the rows covers their slots up to a whole block of 128.
+    for nx in (2, 254, 256, 258, 2 ** 31 - 2, 2 ** 31 - 256, 2 ** 31 - 258):
+        for k in [0, 1] + list(range(max(0, nx // 2 - 2), -(-nx // 2 // 128) * 128 + 128)):
+            yield nx, 1, k, 2, (2 * k if k < nx // 2 else 0, int(k < nx // 2), 0)
 
 
 def test_slots_of_every_box_the_library_accepts(tmp_path):
