@@ -277,12 +277,12 @@ const char *flbm_last_error(void);
 
 /*
  * Batched ensembles: many independent periodic lattices, each with its own lattice
- * type, size, relaxation rates, kBT, rho0 and noise seed, advanced together by one
- * persistent kernel launch per flbm_batch_step call. Every lattice follows exactly the
+ * type, size, relaxation rates, kBT, rho0 and noise seed, advanced together by the launches
+ * of a flbm_batch_step call (flbm_batch_set_shape). Every lattice follows exactly the
  * update of a single context with the same parameters (the same Philox stream keyed on
  * its own seed, step and site); only the launch shape differs. The paper itself runs one
  * lattice at a time; ensembles of independent runs are how its fluctuation statistics
- * are gathered (Sec. III), which this form does in one launch.
+ * are gathered (Sec. III), which this form does together.
  *
  * One spec per lattice (plain data, copied by flbm_batch_create):
  *   lattice, dims, lambda, kBT, rho0, seed : as for flbm_create (lambda holds Q rates).
